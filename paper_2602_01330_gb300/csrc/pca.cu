@@ -6,12 +6,13 @@
 // * Covariance C = Z^T Z / (m - 1): 32 x 32 output tiles, the standardised rows staged in
 //   shared memory 32 at a time, FP32 accumulation.
 // * Eigenvectors: parallel cyclic Jacobi (round-robin pairing: every round rotates p/2
-//   disjoint index pairs, a sweep is p - 1 rounds). A round is two launches: the rotation
-//   angles of all pairs from the current matrix, then one thread per 2 x 2 block (i1, j1) x
-//   (i2, j2) applying both rotations at once, J1^T B J2, so rows and columns move together;
-//   the eigenvector matrix is kept transposed (row i = eigenvector i), so its update is a
-//   row update. A fixed number of sweeps runs without host synchronisation; the remaining
-//   relative off-diagonal norm is returned.
+//   disjoint index pairs, a sweep is p - 1 rounds). Each 2 x 2 block (i1, j1) x (i2, j2) takes
+//   both rotations at once, J1^T B J2, so rows and columns move together; the eigenvector
+//   matrix is kept transposed (row i = eigenvector i), so its update is a row update. All
+//   rounds run in one cooperative launch with the matrix in shared memory
+//   (jacobi_persist_kernel) as long as it fits, one launch per round beyond. A fixed number of
+//   sweeps runs without host synchronisation; the remaining relative off-diagonal norm is
+//   returned.
 // * Selection: eigenvalues ranked in decreasing order (the smaller index first on ties), the
 //   leading k rows written with the sign that makes the entry of largest magnitude positive.
 // * Transform: y = ((x - mean) / scale) C_k^T by 32 x 32 tiles; min-max scaling fitted on
@@ -109,6 +110,50 @@ __global__ void eye_kernel(float* __restrict__ Vt, int p) {
 // index of round-robin position t in round r (positions 0..pe-1, pe even; 0 stays put)
 __device__ __forceinline__ int rr_pos(int t, int r, int pe) { return t == 0 ? 0 : 1 + (t - 1 + r) % (pe - 1); }
 
+// (c, s, t) of the rotation that zeroes a_ij, i < j
+__device__ __forceinline__ float4 pair_rotation(float aii, float ajj, float aij) {
+  float c = 1.0f, s = 0.0f, t = 0.0f;
+  if (fabsf(aij) > 1e-30f) {
+    // angle that zeroes a_ij: tau = (a_jj - a_ii) / (2 a_ij), t the smaller root
+    const float tau = (ajj - aii) / (2.0f * aij);
+    t = (tau >= 0.0f ? 1.0f : -1.0f) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
+    c = __frsqrt_rn(1.0f + t * t);  // correctly rounded: c^2 + s^2 - 1 stays unbiased
+    s = t * c;
+  }
+  return make_float4(c, s, t, 0.0f);
+}
+
+// B' = J1^T B J2 of one 2 x 2 block (J = [[c, s], [-s, c]]); `own`: the block of a pair with
+// itself, whose rotation zeroes the off-diagonal and moves the diagonal by -/+ t a_ij, which
+// keeps the trace to one rounding
+__device__ __forceinline__ void rotate_block(float4 r1, float4 r2, bool own, float& b00, float& b01, float& b10,
+                                             float& b11) {
+  // explicit fmaf: the same bits wherever a block or one of its elements is computed
+  // rows: R0 = c1 B0 - s1 B1, R1 = s1 B0 + c1 B1
+  const float q00 = fmaf(r1.x, b00, -__fmul_rn(r1.y, b10)), q01 = fmaf(r1.x, b01, -__fmul_rn(r1.y, b11));
+  const float q10 = fmaf(r1.y, b00, __fmul_rn(r1.x, b10)), q11 = fmaf(r1.y, b01, __fmul_rn(r1.x, b11));
+  // columns: C0 = c2 R.0 - s2 R.1, C1 = s2 R.0 + c2 R.1
+  float n00 = fmaf(r2.x, q00, -__fmul_rn(r2.y, q01)), n01 = fmaf(r2.y, q00, __fmul_rn(r2.x, q01));
+  float n10 = fmaf(r2.x, q10, -__fmul_rn(r2.y, q11)), n11 = fmaf(r2.y, q10, __fmul_rn(r2.x, q11));
+  if (own) {
+    n00 = fmaf(-r1.z, b01, b00);
+    n11 = fmaf(r1.z, b01, b11);
+    n01 = 0.0f;
+    n10 = 0.0f;
+  }
+  b00 = n00;
+  b01 = n01;
+  b10 = n10;
+  b11 = n11;
+}
+
+// rows i, j of V^T under the pair's rotation
+__device__ __forceinline__ void rotate_rows(float c, float s, float& u, float& v) {
+  const float a = fmaf(c, u, -__fmul_rn(s, v)), b = fmaf(s, u, __fmul_rn(c, v));
+  u = a;
+  v = b;
+}
+
 // rotation angles of pair k of round r: (i, j, c, s) with i < j; a pair holding the
 // padding index p (odd p) is the identity
 __device__ __forceinline__ void jacobi_pair_params(const float* A, int p, int pe, int r, int k, int2* ij,
@@ -119,19 +164,9 @@ __device__ __forceinline__ void jacobi_pair_params(const float* A, int p, int pe
     i = j;
     j = t;
   }
-  float c = 1.0f, s = 0.0f, t = 0.0f;
-  if (j < p) {
-    const float aii = A[(long long)i * p + i], ajj = A[(long long)j * p + j], aij = A[(long long)i * p + j];
-    if (fabsf(aij) > 1e-30f) {
-      // angle that zeroes a_ij: tau = (a_jj - a_ii) / (2 a_ij), t the smaller root
-      const float tau = (ajj - aii) / (2.0f * aij);
-      t = (tau >= 0.0f ? 1.0f : -1.0f) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
-      c = __frsqrt_rn(1.0f + t * t);  // correctly rounded: c^2 + s^2 - 1 stays unbiased
-      s = t * c;
-    }
-  }
   ij[k] = make_int2(i, j);
-  cs[k] = make_float4(c, s, t, 0.0f);
+  cs[k] = j < p ? pair_rotation(A[(long long)i * p + i], A[(long long)j * p + j], A[(long long)i * p + j])
+                : make_float4(1.0f, 0.0f, 0.0f, 0.0f);
 }
 
 // the rotation angles of round r (the first round of a fit)
@@ -162,34 +197,22 @@ __global__ void __launch_bounds__(256) jacobi_rotate_kernel(float* __restrict__ 
     const float4 r2 = cs[k2];
     const int i2 = b.x, j2 = b.y;
     const bool has_j2 = j2 < p;
-    const float b00 = A[(long long)i1 * p + i2];
-    const float b01 = has_j2 ? A[(long long)i1 * p + j2] : 0.0f;
-    const float b10 = has_j1 ? A[(long long)j1 * p + i2] : 0.0f;
-    const float b11 = (has_j1 && has_j2) ? A[(long long)j1 * p + j2] : 0.0f;
-    // rows: R0 = c1 B0 - s1 B1, R1 = s1 B0 + c1 B1
-    const float q00 = r1.x * b00 - r1.y * b10, q01 = r1.x * b01 - r1.y * b11;
-    const float q10 = r1.y * b00 + r1.x * b10, q11 = r1.y * b01 + r1.x * b11;
-    // columns: C0 = c2 R.0 - s2 R.1, C1 = s2 R.0 + c2 R.1
-    float n00 = r2.x * q00 - r2.y * q01, n01 = r2.y * q00 + r2.x * q01;
-    float n10 = r2.x * q10 - r2.y * q11, n11 = r2.y * q10 + r2.x * q11;
-    if (k1 == k2 && has_j1) {
-      // the pair's own block: the rotation zeroes its off-diagonal, and the diagonal moves
-      // by -/+ t a_ij, which keeps the trace to one rounding
-      n00 = b00 - r1.z * b01;
-      n11 = b11 + r1.z * b01;
-      n01 = 0.0f;
-      n10 = 0.0f;
-    }
-    A[(long long)i1 * p + i2] = n00;
-    if (has_j2) A[(long long)i1 * p + j2] = n01;
-    if (has_j1) A[(long long)j1 * p + i2] = n10;
-    if (has_j1 && has_j2) A[(long long)j1 * p + j2] = n11;
+    float b00 = A[(long long)i1 * p + i2];
+    float b01 = has_j2 ? A[(long long)i1 * p + j2] : 0.0f;
+    float b10 = has_j1 ? A[(long long)j1 * p + i2] : 0.0f;
+    float b11 = (has_j1 && has_j2) ? A[(long long)j1 * p + j2] : 0.0f;
+    rotate_block(r1, r2, k1 == k2 && has_j1, b00, b01, b10, b11);
+    A[(long long)i1 * p + i2] = b00;
+    if (has_j2) A[(long long)i1 * p + j2] = b01;
+    if (has_j1) A[(long long)j1 * p + i2] = b10;
+    if (has_j1 && has_j2) A[(long long)j1 * p + j2] = b11;
   }
   if (has_j1) {
     for (int col = threadIdx.x; col < p; col += blockDim.x) {
-      const float u = Vt[(long long)i1 * p + col], v = Vt[(long long)j1 * p + col];
-      Vt[(long long)i1 * p + col] = r1.x * u - r1.y * v;
-      Vt[(long long)j1 * p + col] = r1.y * u + r1.x * v;
+      float u = Vt[(long long)i1 * p + col], v = Vt[(long long)j1 * p + col];
+      rotate_rows(r1.x, r1.y, u, v);
+      Vt[(long long)i1 * p + col] = u;
+      Vt[(long long)j1 * p + col] = v;
     }
   }
   if (r_next < 0) return;
@@ -204,15 +227,422 @@ __global__ void __launch_bounds__(256) jacobi_rotate_kernel(float* __restrict__ 
   if (threadIdx.x == 0) *done = 0u;
 }
 
-// sqrt(off-diagonal sum of squares / total sum of squares) of A
-__global__ void __launch_bounds__(256) off_norm_kernel(const float* __restrict__ A, int p, float* __restrict__ out) {
-  double off = 0.0, all = 0.0;
-  const long long n = (long long)p * p;
-  for (long long e = threadIdx.x; e < n; e += 256) {
-    const double v = A[e];
-    all += v * v;
-    if (e / p != e % p) off += v * v;
+// ---- the same rounds in one launch, the matrix held in shared memory ----
+//
+// A round of the launch-per-round form is a few hundred nanoseconds of arithmetic inside 10 us
+// of launch, scattered reads and a last-CTA pass. Here one cooperative launch runs every round:
+//  * Round-robin positions are a ring: with position 0 fixed, the index at position t moves to
+//    t - 1 each round (1 to pe - 1). Pair k holds positions (k, pe - 1 - k). CTA g owns `ppc`
+//    consecutive pairs, i.e. the rows of A at 2 ppc positions, whole, in shared memory; per
+//    round one row of its upper run goes to CTA g - 1 and one of its lower run to g + 1.
+//  * The angle of a pair needs a_ii, a_jj and a_ij. A diagonal element changes only with its own
+//    pair's rotation, so every CTA keeps the whole diagonal; the owner of row i computes the
+//    pair's a_ij of the next round and its angle first of all and publishes them. A round then
+//    costs one trip through L2, under which the rows and the columns of V^T are rotated. V^T is
+//    split by columns, which rotations never mix.
+//  * Rows stand at their positions in two copies: a round reads one and writes the other, each
+//    row where it stands next, so one barrier a round is enough.
+//  * Everything in transit is a 16-byte word with a round tag, stored and loaded as one: the tag
+//    says that the values are there, so there is no barrier and no fence. Words alternate
+//    between two buffers; a word of round q + 2 is written only after its CTA has read every
+//    angle of round q + 1, i.e. after every CTA has read those of round q. All waits are
+//    bounded; the launch is cooperative, so the CTAs run at the same time.
+// Up to about 130 features everything fits one CTA, and the angles pass through shared memory.
+// The arithmetic and its order are those of jacobi_rotate_kernel: bit-identical results.
+// Bound by the latency of a round: the L2 round trip (about 950 cycles from a store to another
+// SM's load of it), the angle's divisions and roots (about 700 on one warp) and one barrier.
+// Measured, 10 sweeps at p = 784 (131 CTAs of 3 row pairs): 13.2 ms, 1.7 us a round, against
+// 79.4 ms with one launch per round (10.1 us).
+
+constexpr int UR = 4;  // row pairs of a thread in flight
+
+struct PersistPlan {
+  int ctas, ppc, vc, threads;  // vc: columns of V^T per CTA
+  size_t smem, box_bytes;
+};
+
+// Box memory (16-byte words): for several CTAs the rows in transit (2 buffers x CTAs x 2 rows x
+// np column pairs), then the published angles (2 buffers x pe). It ends with V^T's part of the
+// workspace, which is written only at the end, and reaches back into A's: the first row is
+// sent in round 0 by a CTA that has everybody's angles, i.e. after every CTA has read its part
+// of A. The fewest pairs per CTA that this and the SM count allow: a CTA's work on its rows is
+// what a round waits for.
+inline PersistPlan persist_plan(int p, int sms, size_t box_cap, size_t angle_cap) {
+  const int pe = p + (p & 1), np = pe / 2;
+  const int lanes = (np + 31) / 32 * 32;  // one thread per column pair, groups of them over the rows
+  constexpr size_t SMEM_CAP = 220 * 1024;
+  auto make = [&](int ppc) {
+    PersistPlan q;
+    q.ppc = ppc;
+    q.ctas = (np + ppc - 1) / ppc;
+    q.vc = (p + q.ctas - 1) / q.ctas;
+    // a thread per column pair, in groups over the row pairs when there are more than UR of
+    // these, and warps of their own for the elements that the next round waits for
+    const int side = (2 * ppc + 31) / 32 * 32, room = (1024 - side) / lanes, want = (ppc + UR - 1) / UR;
+    q.threads = lanes * (room < want ? room : want) + side;
+    q.smem = size_t((q.vc + 3) / 4) * pe * 16 + size_t(2) * np * 16 + size_t(pe) * 16 + size_t(4) * ppc * pe * 4 +
+             size_t(pe) * 4;
+    q.box_bytes = size_t(32) * pe + (q.ctas > 1 ? size_t(32) * q.ctas * pe : 0);
+    return q;
+  };
+  if (np <= 960 && size_t(32) * pe <= angle_cap) {
+    const PersistPlan one = make(np);
+    if (one.smem <= SMEM_CAP) return one;
+    for (int ppc = 2; ppc < np; ++ppc) {
+      const PersistPlan q = make(ppc);
+      if (q.ctas > 1 && q.ctas <= sms && q.smem <= SMEM_CAP && q.box_bytes <= box_cap) return q;
+    }
   }
+  return PersistPlan{0, 0, 0, 0, 0, 0};
+}
+
+struct PersistArgs {
+  float* A;
+  float* Vt;
+  uint4* words;  // box memory
+  unsigned* done;
+  unsigned* status;
+  int p, ppc, vc, rounds;
+};
+
+// Round tags are bit patterns of negative signalling NaNs, which no arithmetic result has, so
+// nothing that the workspace held before (the covariance) reads as one.
+__device__ __forceinline__ unsigned tag_of(int round) { return 0xff800001u + unsigned(round); }
+
+__device__ __forceinline__ void put_word(uint4* w, float v0, float v1, float v2, unsigned tag) {
+  asm volatile(
+      "{\n\t.reg .b128 x;\n\t.reg .b64 lo, hi;\n\tmov.b64 lo, {%1, %2};\n\tmov.b64 hi, {%3, %4};\n\t"
+      "mov.b128 x, {lo, hi};\n\tst.relaxed.gpu.global.b128 [%0], x;\n\t}" ::"l"(w),
+      "r"(__float_as_uint(v0)), "r"(__float_as_uint(v1)), "r"(__float_as_uint(v2)), "r"(tag)
+      : "memory");
+}
+__device__ __forceinline__ uint4 get_word(const uint4* w) {
+  unsigned long long lo, hi;
+  asm volatile(
+      "{\n\t.reg .b128 x;\n\tld.relaxed.gpu.global.b128 x, [%2];\n\tmov.b128 {%0, %1}, x;\n\t}"
+      : "=l"(lo), "=l"(hi)
+      : "l"(w)
+      : "memory");
+  return make_uint4(unsigned(lo), unsigned(lo >> 32), unsigned(hi), unsigned(hi >> 32));
+}
+
+// Waits (bounded) until the word at `src` carries `tag`; `w` may hold an earlier look at it. The
+// clock, a slow read, is looked at every 1024 polls.
+__device__ __forceinline__ bool await_word(uint4& w, const uint4* src, unsigned tag) {
+  unsigned long long t0 = 0;
+  for (unsigned it = 1; w.w != tag; ++it) {
+    w = get_word(src);
+    if ((it & 1023u) == 0u) {
+      const unsigned long long t = globaltimer_ns();
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > WAIT_LIMIT_NS) return false;
+    }
+  }
+  return true;
+}
+
+template <int MAXT, bool ODD>
+__global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistArgs a) {
+  constexpr int NR = MAXT > 512 ? 2 : UR;  // row pairs in flight: what the registers hold
+  extern __shared__ __align__(16) float sm[];
+  const int p = a.p, pe = p + (p & 1), np = pe / 2, ring = pe - 1;
+  const int G = int(gridDim.x), g = int(blockIdx.x), NT = int(blockDim.x), tid = int(threadIdx.x);
+  const int ks = g * a.ppc, ke = min(ks + a.ppc, np), cnt = ke - ks;
+  const int v0 = g * a.vc, vn = max(0, min(a.vc, p - v0)), vp = (a.vc + 3) / 4;
+  const bool solo = G == 1;
+  // shared memory: V^T columns [plane][row][4], angles [2 rounds][pair] (c, s, t), solo: the
+  // published angles by x, rows [2 rounds][local row][pe], the diagonal of A
+  float4* V = reinterpret_cast<float4*>(sm);
+  float4* pars = V + vp * pe;
+  float4* sN = pars + 2 * np;
+  float* rows = reinterpret_cast<float*>(sN + pe);
+  float* sD = rows + 4 * a.ppc * pe;
+  __shared__ int s_abort;
+  uint4* wR = a.words;                                              // [buffer][CTA][upper / lower][np]
+  uint4* wN = wR + (solo ? 0 : size_t(4) * G * np);                 // [buffer][pe]
+  auto box = [&](int buf, int cta, int which) { return wR + (size_t(buf * G + cta) * 2 + which) * np; };
+  auto idx_at = [&](int t, int r) {  // index at position t in round r
+    int x = t - 1 + r;
+    if (x >= ring) x -= ring;
+    return t == 0 ? 0 : 1 + x;
+  };
+  auto came_from = [&](int t) { return t == 0 ? 0 : (t == ring ? 1 : t + 1); };  // its position a round earlier
+  auto goes_to = [&](int t) { return t == 0 ? 0 : (t == 1 ? ring : t - 1); };
+  // local row u < cnt: position ks + u; u >= cnt: position pe - ke + (u - cnt)
+  auto pos_of = [&](int u) { return u < cnt ? ks + u : pe - ke + (u - cnt); };
+  auto row_at = [&](int t) { return t < np ? t - ks : cnt + t - (pe - ke); };
+  // where local row u stands next; -1: at another CTA
+  auto moves_to = [&](int u) {
+    const int t = goes_to(pos_of(u));
+    return ((t >= ks && t < ke) || (t >= pe - ke && t < pe - ks)) ? row_at(t) : -1;
+  };
+
+  for (int e = tid; e < 2 * cnt * pe; e += NT) {
+    const int u = e / pe, c = e - u * pe, i = pos_of(u);
+    rows[e] = (i < p && c < p) ? a.A[(long long)i * p + c] : 0.0f;
+    rows[2 * a.ppc * pe + e] = 0.0f;  // column p of an odd p stays zero
+  }
+  for (int i = tid; i < p; i += NT) sD[i] = a.A[(long long)i * p + i];
+  for (int e = tid; e < vp * pe; e += NT) {
+    const int pl = e / pe, i = e - pl * pe, c = v0 + 4 * pl;
+    V[e] = make_float4(c == i ? 1.0f : 0.0f, c + 1 == i ? 1.0f : 0.0f, c + 2 == i ? 1.0f : 0.0f,
+                       c + 3 == i ? 1.0f : 0.0f);
+  }
+  if (tid == 0) s_abort = 0;
+  __syncthreads();  // what this CTA reads of A is read: only now does it publish anything
+  for (int u = tid; u < 2 * cnt; u += NT) {
+    const int i = pos_of(u), j = ring - i;  // round 0: index = position
+    if (i < j && j < p) {
+      const float o = rows[u * pe + j];
+      const float4 w = pair_rotation(sD[i], sD[j], o);
+      if (solo) sN[i] = make_float4(w.x, w.z, o, 0.0f);
+      else put_word(wN + i, w.x, w.z, o, tag_of(0));
+    }
+  }
+  __syncthreads();
+
+  const int side = (2 * a.ppc + 31) / 32 * 32, workers = NT - side;
+  const int copy = 2 * a.ppc * pe;  // floats between the two copies of the rows
+  const bool can_up = g < G - 1, can_low = g > 0;
+  if (tid >= workers) {
+    // ---- the next round's elements and angles: row u's partner is at position ty, that one's at ring - ty ----
+    const int u = tid - workers;
+    const bool holds = u < 2 * cnt;
+    const int hu = holds ? (u < cnt ? u : 2 * cnt - 1 - u) : 0;
+    const int ty = holds ? came_from(ring - goes_to(pos_of(u))) : 0, kc = min(ty, ring - ty);
+    int r = 0;
+    for (int q = 0; q < a.rounds; ++q) {
+      const int buf = q & 1;
+      const int x = holds ? idx_at(pos_of(u), r) : 0, y = idx_at(ty, r), z = idx_at(ring - ty, r);
+      const bool up = idx_at(ks + hu, r) < idx_at(ring - ks - hu, r), low = y < z;
+      const float* ri = rows + buf * copy + (up ? hu : 2 * cnt - 1 - hu) * pe;
+      const float* rj = rows + buf * copy + (up ? 2 * cnt - 1 - hu : hu) * pe;
+      const int c0 = low ? y : z, c1 = low ? z : y;
+      const bool is_i = (u < cnt) == up;
+      __syncthreads();
+      if (s_abort) break;
+      if (q + 1 < a.rounds && holds && y > x && y < p) {  // otherwise the partner's owner does it
+        float b00 = ri[c0], b01 = ri[c1], b10 = rj[c0], b11 = rj[c1];
+        rotate_block(pars[buf * np + ks + hu], pars[buf * np + kc], ks + hu == kc, b00, b01, b10, b11);
+        const float o = is_i ? (low ? b00 : b01) : (low ? b10 : b11);
+        const float4 w = pair_rotation(sD[x], sD[y], o);
+        if (solo) sN[x] = make_float4(w.x, w.z, o, 0.0f);
+        else put_word(wN + (buf ^ 1) * pe + x, w.x, w.z, o, tag_of(q + 1));
+      }
+      if (++r == ring) r = 0;
+      if (solo) __syncthreads();
+    }
+  } else {
+    // ---- column pair k2 and, NR at a time, the row pairs grp, grp + groups, ... of an order that
+    // takes the two with a row to send first ----
+    const int lanes = (np + 31) / 32 * 32;
+    int groups = workers / lanes, grp = tid / lanes, k2 = tid - grp * lanes;
+    asm volatile("" : "+r"(groups), "+r"(grp), "+r"(k2));  // opaque: not to be divided again in every round
+    const bool active = k2 < np;
+    auto turn = [&](int n) { return n == 0 ? 0 : (n == 1 ? cnt - 1 : n - 1); };
+    // what stays the same in every round, for the first NR row pairs: where the rows stand and go
+    // (floats; -1: sent away), and the rounds [first, first + len) in which the lower position
+    // holds the smaller index
+    const bool once = cnt <= NR * groups;
+    int st_u[NR], st_ou[NR], st_ol[NR], st_du[NR], st_dl[NR], st_f[NR], st_len[NR];
+    auto set_turn = [&](int z, int n) {
+      const int u = turn(n), t = ks + u;
+      st_u[z] = u;
+      st_ou[z] = u * pe;
+      st_ol[z] = (2 * cnt - 1 - u) * pe;
+      const int du = moves_to(u), dl = moves_to(2 * cnt - 1 - u);
+      st_du[z] = du < 0 ? -1 : du * pe;
+      st_dl[z] = dl < 0 ? -1 : dl * pe;
+      st_f[z] = t + 1;
+      st_len[z] = t == 0 ? 0 : ring - 2 * t;
+    };
+#pragma unroll
+    for (int z = 0; z < NR; ++z) set_turn(z, min(grp + z * groups, cnt - 1));
+    uint4* in_up = box(0, g, 0) + k2;
+    uint4* in_low = box(0, g, 1) + k2;
+    uint4* out_up = can_low ? box(0, g - 1, 0) + k2 : nullptr;   // the row at position ks
+    uint4* out_low = can_up ? box(0, g + 1, 1) + k2 : nullptr;   // at pe - ke
+    const size_t flip = size_t(2) * G * np;                       // words between the two buffers
+    // the rows in transit: group 0 takes the upper one, and the lower one if it is the only group
+    const bool takes_up = can_up && active && grp == 0, takes_low = can_low && active && grp == (groups > 1 ? 1 : 0);
+    const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+    uint4 wn = none, wu = none, wl = none;  // looks at the next round's angle and row words
+    bool ok = true;
+    int x2 = k2, y2 = active ? ring - k2 : 0;  // the pair's indices: they move up by one each round
+    int xp = 0, yp = 0;
+    int r = 0;
+    for (int q = 0; q < a.rounds; ++q) {
+      const unsigned tag = tag_of(q), next = tag_of(q + 1);
+      const int buf = q & 1;
+      const bool more = q + 1 < a.rounds;
+      float4* par = pars + buf * np;
+      float* cur = rows + buf * copy;
+      float* nxt = rows + (buf ^ 1) * copy;
+      const int i2 = min(x2, y2), j2 = max(x2, y2);
+      const bool has_j2 = !ODD || j2 < p;
+      // 1. every pair's angle, and the whole diagonal after this round; the rows that moved here
+      // (the ends of the upper run, from CTA g + 1, and of the lower one, from g - 1)
+      float4 r2 = make_float4(1.0f, 0.0f, 0.0f, 0.0f);
+      if (grp == 0 && active) {
+        if (has_j2) {
+          float o;
+          if (solo) {
+            const float4 v = sN[i2];
+            r2.x = v.x;
+            r2.z = v.y;
+            o = v.z;
+          } else {
+            ok = await_word(wn, wN + buf * pe + i2, tag) && ok;
+            r2.x = __uint_as_float(wn.x);
+            r2.z = __uint_as_float(wn.y);
+            o = __uint_as_float(wn.z);
+          }
+          r2.y = r2.z * r2.x;
+          sD[i2] = fmaf(-r2.z, o, sD[i2]);  // the pair's own block in rotate_block
+          sD[j2] = fmaf(r2.z, o, sD[j2]);
+        }
+        par[k2] = r2;
+      }
+      if (q > 0) {
+        const int ip = min(xp, yp), jp = max(xp, yp);  // the columns of pair k2 in the round that sent them
+        if (takes_up) {
+          ok = await_word(wu, in_up + buf * flip, tag) && ok;
+          cur[(cnt - 1) * pe + ip] = __uint_as_float(wu.x);
+          if (!ODD || jp < p) cur[(cnt - 1) * pe + jp] = __uint_as_float(wu.y);
+        }
+        if (takes_low) {
+          ok = await_word(wl, in_low + buf * flip, tag) && ok;
+          cur[(2 * cnt - 1) * pe + ip] = __uint_as_float(wl.x);
+          if (!ODD || jp < p) cur[(2 * cnt - 1) * pe + jp] = __uint_as_float(wl.y);
+        }
+      }
+      if (!ok) s_abort = 1;
+      __syncthreads();
+      if (s_abort) break;
+      // 2. this CTA's rows
+      if (grp != 0 && active) r2 = par[k2];
+      if (active) {
+        for (int n0 = grp; n0 < cnt; n0 += NR * groups) {
+          if (!once) {
+#pragma unroll
+            for (int z = 0; z < NR; ++z) set_turn(z, min(n0 + z * groups, cnt - 1));
+          }
+          float b[NR][4];
+          float4 r1[NR];
+#pragma unroll
+          for (int z = 0; z < NR; ++z) {
+            if (n0 + z * groups < cnt) {
+              const bool up = unsigned(r - st_f[z]) >= unsigned(st_len[z]);  // the upper position holds i
+              const float* ri = cur + (up ? st_ou[z] : st_ol[z]);
+              const float* rj = cur + (up ? st_ol[z] : st_ou[z]);
+              r1[z] = par[ks + st_u[z]];
+              b[z][0] = ri[i2];
+              b[z][1] = ri[j2];
+              b[z][2] = rj[i2];
+              b[z][3] = rj[j2];
+            }
+          }
+#pragma unroll
+          for (int z = 0; z < NR; ++z) {
+            if (n0 + z * groups < cnt) {
+              const int u = st_u[z];
+              const bool up = unsigned(r - st_f[z]) >= unsigned(st_len[z]);
+              rotate_block(r1[z], r2, ks + u == k2 && has_j2, b[z][0], b[z][1], b[z][2], b[z][3]);
+              if (ODD && max(idx_at(ks + u, r), idx_at(ring - ks - u, r)) == p) b[z][2] = b[z][3] = 0.0f;  // no such row
+              const float u0 = up ? b[z][0] : b[z][2], u1 = up ? b[z][1] : b[z][3];  // the upper row's values
+              const float l0 = up ? b[z][2] : b[z][0], l1 = up ? b[z][3] : b[z][1];
+              if (more) {
+                if (st_du[z] >= 0) {
+                  nxt[st_du[z] + i2] = u0;
+                  if (has_j2) nxt[st_du[z] + j2] = u1;
+                } else {
+                  put_word(out_up + (buf ^ 1) * flip, u0, u1, 0.0f, next);
+                }
+                if (st_dl[z] >= 0) {
+                  nxt[st_dl[z] + i2] = l0;
+                  if (has_j2) nxt[st_dl[z] + j2] = l1;
+                } else {
+                  put_word(out_low + (buf ^ 1) * flip, l0, l1, 0.0f, next);
+                }
+              } else {  // the last round's rows stay where they are
+                nxt[st_ou[z] + i2] = u0;
+                if (has_j2) nxt[st_ou[z] + j2] = u1;
+                nxt[st_ol[z] + i2] = l0;
+                if (has_j2) nxt[st_ol[z] + j2] = l1;
+              }
+            }
+          }
+        }
+        // 3. this CTA's columns of V^T
+        if (has_j2) {
+#pragma unroll 2
+          for (int pl = grp; pl < vp; pl += groups) {
+            float4 u = V[pl * pe + i2], v = V[pl * pe + j2];
+            rotate_rows(r2.x, r2.y, u.x, v.x);
+            rotate_rows(r2.x, r2.y, u.y, v.y);
+            rotate_rows(r2.x, r2.y, u.z, v.z);
+            rotate_rows(r2.x, r2.y, u.w, v.w);
+            V[pl * pe + i2] = u;
+            V[pl * pe + j2] = v;
+          }
+        }
+        // 4. the pair's indices in the next round, and a first look at its words
+        xp = x2;
+        yp = y2;
+        if (x2 != 0) x2 = x2 == ring ? 1 : x2 + 1;  // position 0 keeps index 0
+        y2 = y2 == ring ? 1 : y2 + 1;
+        if (!solo && more) {
+          if (grp == 0) wn = get_word(wN + (buf ^ 1) * pe + min(x2, y2));
+          if (takes_up) wu = get_word(in_up + (buf ^ 1) * flip);
+          if (takes_low) wl = get_word(in_low + (buf ^ 1) * flip);
+        }
+      }
+      if (++r == ring) r = 0;
+      if (solo) __syncthreads();  // the next angles are in shared memory
+    }
+  }
+
+  // every CTA has read its last words before the memory that holds them is written
+  __syncthreads();
+  if (!solo) {
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(a.done, 1u);
+      const unsigned long long t0 = globaltimer_ns();
+      while (*reinterpret_cast<volatile unsigned*>(a.done) < unsigned(G))
+        if (globaltimer_ns() - t0 > WAIT_LIMIT_NS) {
+          s_abort = 1;
+          break;
+        }
+    }
+    __syncthreads();
+  }
+  if (s_abort) {
+    if (tid == 0) record_status(a.status, DEV_TIMEOUT);
+    return;
+  }
+  const int rl = (a.rounds - 1) % ring;  // rows stand where the last round had them
+  const float* last = rows + (a.rounds & 1) * copy;
+  for (int e = tid; e < 2 * cnt * p; e += NT) {
+    const int u = e / p, c = e - u * p, i = idx_at(pos_of(u), rl);
+    if (i < p) a.A[(long long)i * p + c] = last[u * pe + c];
+  }
+  for (int e = tid; e < p * vn; e += NT) {
+    const int i = e / vn, c = e - i * vn;
+    a.Vt[(long long)i * p + v0 + c] = reinterpret_cast<const float*>(V + (c >> 2) * pe + i)[c & 3];
+  }
+}
+
+// sqrt(off-diagonal sum of squares / total sum of squares) of A: CTA b sums the rows b, b + grid,
+// ... into part[b] (off-diagonal, total); the finish adds the parts in order
+__global__ void __launch_bounds__(256) off_norm_kernel(const float* __restrict__ A, int p, double2* __restrict__ part) {
+  double off = 0.0, all = 0.0;
+  for (int i = blockIdx.x; i < p; i += gridDim.x)
+    for (int c = threadIdx.x; c < p; c += 256) {
+      const double v = A[(long long)i * p + c], v2 = v * v;
+      all += v2;
+      if (c != i) off += v2;
+    }
   __shared__ double s_off[256], s_all[256];
   s_off[threadIdx.x] = off;
   s_all[threadIdx.x] = all;
@@ -224,7 +654,22 @@ __global__ void __launch_bounds__(256) off_norm_kernel(const float* __restrict__
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) *out = s_all[0] > 0.0 ? float(sqrt(s_off[0] / s_all[0])) : 0.0f;
+  if (threadIdx.x == 0) part[blockIdx.x] = make_double2(s_off[0], s_all[0]);
+}
+
+__global__ void __launch_bounds__(32) off_norm_finish_kernel(const double2* __restrict__ part, int n,
+                                                             float* __restrict__ out) {
+  double off = 0.0, all = 0.0;
+  for (int e = threadIdx.x; e < n; e += 32) {
+    off += part[e].x;
+    all += part[e].y;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    off += __shfl_xor_sync(0xffffffffu, off, o);
+    all += __shfl_xor_sync(0xffffffffu, all, o);
+  }
+  if (threadIdx.x == 0) *out = all > 0.0 ? float(sqrt(off / all)) : 0.0f;
 }
 
 // block i: the rank of eigenvalue A_ii among all (decreasing, smaller index first on ties);
@@ -375,17 +820,45 @@ dk_status fit(dk_ctx* ctx, const float* x, int m, int p, int k, int sweeps, cons
               float* scale, float* comps, float* eig, float* off_norm, cudaStream_t st) {
   col_stats_kernel<<<(p + 31) / 32, 256, 0, st>>>(x, m, p, mean, scale);
   cov_kernel<<<dim3((p + T32 - 1) / T32, (p + T32 - 1) / T32), 256, 0, st>>>(x, m, p, mean, scale, w.A);
-  const int fill_blocks = int(((long long)p * p + 255) / 256 < 4096 ? ((long long)p * p + 255) / 256 : 4096);
-  eye_kernel<<<fill_blocks, 256, 0, st>>>(w.Vt, p);
-  const int pe = p + (p & 1), np = pe / 2;
+  const int pe = p + (p & 1), np = pe / 2, rounds = sweeps * (pe - 1);
+  const size_t mat_bytes = round256(size_t(p) * p * sizeof(float));
+  const PersistPlan plan = persist_plan(p, ctx->sm_count, 2 * mat_bytes, mat_bytes);
   if (cudaMemsetAsync(w.done, 0, sizeof(unsigned), st) != cudaSuccess) return DK_ERR_CUDA;
-  jacobi_params_kernel<<<(np + 255) / 256, 256, 0, st>>>(w.A, p, pe, 0, w.ij, w.cs);
-  const int rounds = sweeps * (pe - 1);
-  for (int q = 0; q < rounds; ++q) {
-    const int r_next = q + 1 < rounds ? (q + 1) % (pe - 1) : -1;
-    jacobi_rotate_kernel<<<np, 256, 0, st>>>(w.A, w.Vt, p, np, w.ij, w.cs, w.done, pe, r_next);
+  bool persistent = false;
+  if (plan.ctas > 0) {
+    // no word of V^T's part, which a former call may have used, has a tag yet
+    if (cudaMemsetAsync(w.Vt, 0, mat_bytes, st) != cudaSuccess) return DK_ERR_CUDA;
+    uint8_t* box = reinterpret_cast<uint8_t*>(w.Vt) + mat_bytes - plan.box_bytes;
+    const bool odd = p & 1, small = plan.threads <= 512;
+    const void* kern = odd ? (small ? reinterpret_cast<const void*>(jacobi_persist_kernel<512, true>)
+                                    : reinterpret_cast<const void*>(jacobi_persist_kernel<1024, true>))
+                           : (small ? reinterpret_cast<const void*>(jacobi_persist_kernel<512, false>)
+                                    : reinterpret_cast<const void*>(jacobi_persist_kernel<1024, false>));
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(plan.smem)) != cudaSuccess)
+      return DK_ERR_CUDA;
+    PersistArgs a{w.A,  w.Vt, reinterpret_cast<uint4*>(box), w.done, ctx->status, p, plan.ppc, plan.vc,
+                  rounds};
+    void* args[] = {&a};
+    persistent = cudaLaunchCooperativeKernel(kern, dim3(plan.ctas), dim3(plan.threads), args, plan.smem, st) ==
+                 cudaSuccess;
+    if (!persistent) cudaGetLastError();  // a device that cannot hold all CTAs at once
   }
-  if (off_norm) off_norm_kernel<<<1, 256, 0, st>>>(w.A, p, off_norm);
+  if (!persistent) {
+    // beyond what shared memory holds: one launch per round
+    const int fill_blocks = int(((long long)p * p + 255) / 256 < 4096 ? ((long long)p * p + 255) / 256 : 4096);
+    eye_kernel<<<fill_blocks, 256, 0, st>>>(w.Vt, p);
+    jacobi_params_kernel<<<(np + 255) / 256, 256, 0, st>>>(w.A, p, pe, 0, w.ij, w.cs);
+    for (int q = 0; q < rounds; ++q) {
+      const int r_next = q + 1 < rounds ? (q + 1) % (pe - 1) : -1;
+      jacobi_rotate_kernel<<<np, 256, 0, st>>>(w.A, w.Vt, p, np, w.ij, w.cs, w.done, pe, r_next);
+    }
+  }
+  if (off_norm) {
+    // the rotation table is done with: it holds the partial sums, one 16-byte entry per CTA
+    double2* part = reinterpret_cast<double2*>(w.cs);
+    off_norm_kernel<<<np, 256, 0, st>>>(w.A, p, part);
+    off_norm_finish_kernel<<<1, 32, 0, st>>>(part, np, off_norm);
+  }
   select_kernel<<<p, 256, 0, st>>>(w.A, w.Vt, p, k, comps, eig);
   return launch_status();
 }

@@ -20,8 +20,8 @@
 // (1 - w) K_c and log K_q are written back (K_c is read from the block, or recomputed with
 // the Gram kernels' compensated feature sum). Entries with K_q <= tau keep their values.
 //
-// Bond 4 and 8: one thread per pair, E in registers, hits queued per warp so that the
-// chains run 32 at a time. Bond 32: one warp per pair, E, the intermediate F and the two
+// Bond 4 and 8: one lane per element of E (8 or 32 lanes per chain), hits queued per warp so
+// that the lanes stay full. Bond 32: one warp per pair, E, the intermediate F and the two
 // samples' site blocks in shared memory; each warp tests 32 entries at once and works
 // through the hits among them.
 #include <math.h>
@@ -73,119 +73,125 @@ __device__ __forceinline__ float2 site_elem(const float2* a, int chi, int h, int
   return __ldg(a + (s * h + jc) * chi + l);
 }
 
-// ---------------- bond 4 / 8: one thread per chain ----------------
+// ---------------- bond 4 / 8: 2 H^2 lanes per chain ----------------
+//
+// Lane (s, p, c) of a chain's group holds E_s[p][c]. Per site it forms F(t, s, a, c) = (E_t
+// A_s[t](x_j))[a][c] for a = p and both t from row p of the E_t (shuffles), then its own
+// E'_s[p][c] from the group's F. Every accumulator adds the same products in the same order as
+// one thread running the whole chain would, so the bits do not depend on the split.
+// A chain is latency bound (a product with its exact error takes 11 instructions, 256 of them a
+// site at bond 4) and most calls have few chains: one thread took 7 us a site. Split over 8
+// lanes the total work grows only by 32 shuffles a lane (bond 8: 32 lanes, 64 shuffles), so
+// full queues gain too. Measured, bond 4, 16 sites: norms of the 8000 training samples of a
+// one-row request 110 -> 14 us and its pass 111 -> 17 us; a 2000-sample Gram's pass (1000 hits)
+// 192 -> 56 us and its norms 100 -> 14 us.
 
 template <int H>
-struct ChainE {
-  DW r[2][H][H], i[2][H][H];
-};
+constexpr int LANES = 2 * H * H;  // lanes per chain
 
-// ln|<psi~_i|psi~_j>| by the double-word chain (FP64 result). mi / mj: the two MPS, with
-// sample counts m_i / m_j (site-major layout).
+__device__ __forceinline__ DW shfl_dw(unsigned mask, DW v, int src, int width) {
+  return {__shfl_sync(mask, v.hi, src, width), __shfl_sync(mask, v.lo, src, width)};
+}
+
+// Mask of this lane's group.
+template <int H>
+__device__ __forceinline__ unsigned group_mask() {
+  constexpr int L = LANES<H>;
+  if constexpr (L == 32) return 0xffffffffu;
+  else return ((1u << L) - 1u) << ((threadIdx.x & 31) & ~(L - 1));
+}
+
+// ln|<psi~_i|psi~_j>| by the double-word chain (FP64 result, valid in every lane of the group).
+// mi / mj: the two MPS, with sample counts m_i / m_j (site-major layout).
 template <int H>
 __device__ double chain_half_log(const float2* __restrict__ mi, int m_i, int i, const float2* __restrict__ mj, int m_j,
                                  int j, int n) {
-  constexpr int CHI = 2 * H;
-  ChainE<H> E;
+  constexpr int CHI = 2 * H, L = LANES<H>;
+  const unsigned mask = group_mask<H>();
+  const int gl = threadIdx.x & (L - 1);
+  const int s = gl / (H * H), p = (gl / H) % H, c = gl % H;
+  // column c of block s of sample j and column p of block s of sample i: 2 H complex numbers
+  // each, element t H + b
+  const float4* pj = reinterpret_cast<const float4*>(mj + size_t(j) * (CHI * CHI) + (s * H + c) * CHI);
+  const float4* pi = reinterpret_cast<const float4*>(mi + size_t(i) * (CHI * CHI) + (s * H + p) * CHI);
+  const size_t step_j = size_t(m_j) * (CHI * CHI / 2), step_i = size_t(m_i) * (CHI * CHI / 2);
+  float4 nb[H], nc[H];
 #pragma unroll
-  for (int t = 0; t < 2; ++t)
-#pragma unroll
-    for (int a = 0; a < H; ++a)
-#pragma unroll
-      for (int c = 0; c < H; ++c) E.r[t][a][c] = E.i[t][a][c] = DW{0.0f, 0.0f};
-  E.r[0][0][0] = DW{1.0f, 0.0f};
+  for (int q = 0; q < H; ++q) {
+    nb[q] = __ldg(pj + q);
+    nc[q] = __ldg(pi + q);
+  }
+  DW er{gl == 0 ? 1.0f : 0.0f, 0.0f}, ei{0.0f, 0.0f};
   int e2 = 0;
   for (int k = 0; k < n; ++k) {
-    const float2* ai = mi + (size_t(k) * m_i + i) * (CHI * CHI);
-    const float2* aj = mj + (size_t(k) * m_j + j) * (CHI * CHI);
-    Acc nr[2][H][H], ni[2][H][H];
+    float br[CHI], bi[CHI], cr[CHI], ci[CHI];
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
+    for (int q = 0; q < H; ++q) {
+      br[2 * q] = nb[q].x;
+      bi[2 * q] = nb[q].y;
+      br[2 * q + 1] = nb[q].z;
+      bi[2 * q + 1] = nb[q].w;
+      cr[2 * q] = nc[q].x;
+      ci[2 * q] = nc[q].y;
+      cr[2 * q + 1] = nc[q].z;
+      ci[2 * q + 1] = nc[q].w;
+    }
+    if (k + 1 < n) {  // the next site's tensors arrive under this site's arithmetic
+      pj += step_j;
+      pi += step_i;
 #pragma unroll
-      for (int p = 0; p < H; ++p)
-#pragma unroll
-        for (int c = 0; c < H; ++c) nr[s][p][c] = ni[s][p][c] = Acc{0.0f, 0.0f};
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-#pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        // F = E_t B with B[b][c] = A_s[t](x_j)[b][c] = element (s, c, t H + b) of sample j
-        DW fr[H][H], fi[H][H];
-#pragma unroll
-        for (int c = 0; c < H; ++c) {
-          float br[H], bi[H];
-#pragma unroll
-          for (int b = 0; b < H; ++b) {
-            const float2 v = site_elem(aj, CHI, H, s, c, t * H + b);
-            br[b] = v.x;
-            bi[b] = v.y;
-          }
-#pragma unroll
-          for (int a = 0; a < H; ++a) {
-            Acc xr{0.0f, 0.0f}, xi{0.0f, 0.0f};
-#pragma unroll
-            for (int b = 0; b < H; ++b) {
-              acc_add(xr, E.r[t][a][b], br[b]);
-              acc_add(xr, E.i[t][a][b], -bi[b]);
-              acc_add(xi, E.r[t][a][b], bi[b]);
-              acc_add(xi, E.i[t][a][b], br[b]);
-            }
-            fr[a][c] = acc_get(xr);
-            fi[a][c] = acc_get(xi);
-          }
-        }
-        // E'_s[p][c] += sum_a conj(C[a][p]) F[a][c], C[a][p] = element (s, p, t H + a) of sample i
-#pragma unroll
-        for (int p = 0; p < H; ++p) {
-          float cr[H], ci[H];
-#pragma unroll
-          for (int a = 0; a < H; ++a) {
-            const float2 v = site_elem(ai, CHI, H, s, p, t * H + a);
-            cr[a] = v.x;
-            ci[a] = v.y;
-          }
-#pragma unroll
-          for (int c = 0; c < H; ++c)
-#pragma unroll
-            for (int a = 0; a < H; ++a) {
-              acc_add(nr[s][p][c], fr[a][c], cr[a]);
-              acc_add(nr[s][p][c], fi[a][c], ci[a]);
-              acc_add(ni[s][p][c], fi[a][c], cr[a]);
-              acc_add(ni[s][p][c], fr[a][c], -ci[a]);
-            }
-        }
+      for (int q = 0; q < H; ++q) {
+        nb[q] = __ldg(pj + q);
+        nc[q] = __ldg(pi + q);
       }
     }
-    float mx = 0.0f;
+    DW fr[2], fi[2];
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
+    for (int t = 0; t < 2; ++t) {
+      Acc xr{0.0f, 0.0f}, xi{0.0f, 0.0f};
 #pragma unroll
-      for (int p = 0; p < H; ++p)
+      for (int b = 0; b < H; ++b) {
+        const int src = (t * H + p) * H + b;
+        const DW vr = shfl_dw(mask, er, src, L), vi = shfl_dw(mask, ei, src, L);
+        acc_add(xr, vr, br[t * H + b]);
+        acc_add(xr, vi, -bi[t * H + b]);
+        acc_add(xi, vr, bi[t * H + b]);
+        acc_add(xi, vi, br[t * H + b]);
+      }
+      fr[t] = acc_get(xr);
+      fi[t] = acc_get(xi);
+    }
+    Acc nr{0.0f, 0.0f}, ni{0.0f, 0.0f};
 #pragma unroll
-        for (int c = 0; c < H; ++c) {
-          E.r[s][p][c] = acc_get(nr[s][p][c]);
-          E.i[s][p][c] = acc_get(ni[s][p][c]);
-          mx = fmaxf(mx, fmaxf(fabsf(E.r[s][p][c].hi), fabsf(E.i[s][p][c].hi)));
-        }
-    if (mx > 0.0f && ((k & 3) == 3 || k == n - 1)) {
-      const int e = exponent_of(mx);
-      const float sc = pow2_neg(e);
+    for (int t = 0; t < 2; ++t)
 #pragma unroll
-      for (int s = 0; s < 2; ++s)
+      for (int a = 0; a < H; ++a) {
+        const int src = (s * H + a) * H + c;
+        const DW vr = shfl_dw(mask, fr[t], src, L), vi = shfl_dw(mask, fi[t], src, L);
+        acc_add(nr, vr, cr[t * H + a]);
+        acc_add(nr, vi, ci[t * H + a]);
+        acc_add(ni, vi, cr[t * H + a]);
+        acc_add(ni, vr, -ci[t * H + a]);
+      }
+    er = acc_get(nr);
+    ei = acc_get(ni);
+    if ((k & 3) == 3 || k == n - 1) {
+      float mx = fmaxf(0.0f, fmaxf(fabsf(er.hi), fabsf(ei.hi)));
 #pragma unroll
-        for (int p = 0; p < H; ++p)
-#pragma unroll
-          for (int c = 0; c < H; ++c) {
-            E.r[s][p][c] = DW{E.r[s][p][c].hi * sc, E.r[s][p][c].lo * sc};
-            E.i[s][p][c] = DW{E.i[s][p][c].hi * sc, E.i[s][p][c].lo * sc};
-          }
-      e2 += e;
+      for (int o = L / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(mask, mx, o, L));
+      if (mx > 0.0f) {
+        const int e = exponent_of(mx);
+        const float sc = pow2_neg(e);
+        er = DW{er.hi * sc, er.lo * sc};
+        ei = DW{ei.hi * sc, ei.lo * sc};
+        e2 += e;
+      }
     }
   }
-  const double re =
-      (double(E.r[0][0][0].hi) + double(E.r[0][0][0].lo)) + (double(E.r[1][0][0].hi) + double(E.r[1][0][0].lo));
-  const double im =
-      (double(E.i[0][0][0].hi) + double(E.i[0][0][0].lo)) + (double(E.i[1][0][0].hi) + double(E.i[1][0][0].lo));
+  const DW r0 = shfl_dw(mask, er, 0, L), r1 = shfl_dw(mask, er, H * H, L);
+  const DW i0 = shfl_dw(mask, ei, 0, L), i1 = shfl_dw(mask, ei, H * H, L);
+  const double re = (double(r0.hi) + double(r0.lo)) + (double(r1.hi) + double(r1.lo));
+  const double im = (double(i0.hi) + double(i0.lo)) + (double(i1.hi) + double(i1.lo));
   return half_log_of(re, im, e2);
 }
 
@@ -239,9 +245,8 @@ __device__ __forceinline__ void write_refined(const GramArgs& g, long long at, i
   }
 }
 
-// Each warp tests 32 entries at a time and queues the hits in shared memory; whenever 32
-// are queued every lane takes one, so the chains run with full warps even when the hits
-// are sparse (a lone hit per warp would otherwise cost the warp its whole chain time).
+// Each warp tests 32 entries at a time and queues the hits in shared memory; the groups of the
+// warp take them in turn, and a rest that would leave groups idle waits for the next 32.
 constexpr int SMALL_WARPS = 4;
 
 template <int H>
@@ -249,7 +254,7 @@ __device__ __forceinline__ void refine_one(const RefineArgs& a, int i, int j, lo
   const double lij = chain_half_log<H>(a.mps_r, a.m_r, i, a.mps_c, a.m_c, j, a.g.n);
   const double lii = a.norm_r ? a.norm_r[i] : chain_half_log<H>(a.mps_r, a.m_r, i, a.mps_r, a.m_r, i, a.g.n);
   const double ljj = a.norm_c ? a.norm_c[j] : chain_half_log<H>(a.mps_c, a.m_c, j, a.mps_c, a.m_c, j, a.g.n);
-  write_refined(a.g, at, i, j, 2.0 * lij - lii - ljj);
+  if ((threadIdx.x & (LANES<H> - 1)) == 0) write_refined(a.g, at, i, j, 2.0 * lij - lii - ljj);
 }
 
 // Marks the samples whose ln-norm some entry above tau needs (all entries of the block,
@@ -272,42 +277,27 @@ __global__ void __launch_bounds__(256) mark_kernel(const RefineArgs a) {
 // (none for a symmetric block). Marked samples are queued per warp as in the pass itself.
 template <int H>
 __device__ __forceinline__ void norm_one(const RefineArgs& a, int u) {
-  if (u < a.m_r) a.norm_r[u] = chain_half_log<H>(a.mps_r, a.m_r, u, a.mps_r, a.m_r, u, a.g.n);
-  else a.norm_c[u - a.m_r] = chain_half_log<H>(a.mps_c, a.m_c, u - a.m_r, a.mps_c, a.m_c, u - a.m_r, a.g.n);
+  const bool row = u < a.m_r;
+  const int i = row ? u : u - a.m_r;
+  const double l = row ? chain_half_log<H>(a.mps_r, a.m_r, i, a.mps_r, a.m_r, i, a.g.n)
+                       : chain_half_log<H>(a.mps_c, a.m_c, i, a.mps_c, a.m_c, i, a.g.n);
+  if ((threadIdx.x & (LANES<H> - 1)) == 0) (row ? a.norm_r : a.norm_c)[i] = l;
 }
 
+// one group of lanes per sample: the chains of the marked samples run side by side
 template <int H>
 __global__ void __launch_bounds__(128) norms_small_kernel(const RefineArgs a, int n_units) {
-  __shared__ int q[4][64];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned below = (1u << lane) - 1u;
-  int count = 0;
-  for (int base = (blockIdx.x * 4 + warp) * 32; base < n_units; base += gridDim.x * 4 * 32) {
-    const int u = base + lane;
-    const bool hit = u < n_units && (u < a.m_r ? a.flag_r[u] : a.flag_c[u - a.m_r]) != 0;
-    const unsigned mask = __ballot_sync(0xffffffffu, hit);
-    if (hit) q[warp][count + __popc(mask & below)] = u;
-    count += __popc(mask);
-    __syncwarp();
-    if (count >= 32) {
-      norm_one<H>(a, q[warp][lane]);
-      __syncwarp();
-      const int rest = count - 32;
-      const int t = lane < rest ? q[warp][32 + lane] : 0;
-      __syncwarp();
-      if (lane < rest) q[warp][lane] = t;
-      count = rest;
-      __syncwarp();
-    }
-  }
-  if (lane < count) norm_one<H>(a, q[warp][lane]);
+  constexpr int PER = 128 / LANES<H>;
+  for (int u = blockIdx.x * PER + threadIdx.x / LANES<H>; u < n_units; u += gridDim.x * PER)
+    if ((u < a.m_r ? a.flag_r[u] : a.flag_c[u - a.m_r]) != 0) norm_one<H>(a, u);
 }
 
 template <int H>
 __global__ void __launch_bounds__(SMALL_WARPS * 32) refine_small_kernel(const RefineArgs a) {
+  constexpr int GROUPS = 32 / LANES<H>;
   __shared__ int qi[SMALL_WARPS][64], qj[SMALL_WARPS][64];
   __shared__ long long qa[SMALL_WARPS][64];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LANES<H>;
   const GramArgs& g = a.g;
   const long long total = (long long)g.nrows * g.ncols;
   const long long nwarps = (long long)gridDim.x * SMALL_WARPS;
@@ -334,28 +324,29 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32) refine_small_kernel(const Re
     }
     count += __popc(mask);
     __syncwarp();
-    if (count >= 32) {
-      refine_one<H>(a, qi[warp][lane], qj[warp][lane], qa[warp][lane]);
-      __syncwarp();
-      const int rest = count - 32;
-      int ti = 0, tj = 0;
-      long long ta = 0;
-      if (lane < rest) {
-        ti = qi[warp][32 + lane];
-        tj = qj[warp][32 + lane];
-        ta = qa[warp][32 + lane];
-      }
-      __syncwarp();
-      if (lane < rest) {
-        qi[warp][lane] = ti;
-        qj[warp][lane] = tj;
-        qa[warp][lane] = ta;
-      }
-      count = rest;
+    int done = 0;
+    for (; done + GROUPS <= count; done += GROUPS) {
+      refine_one<H>(a, qi[warp][done + grp], qj[warp][done + grp], qa[warp][done + grp]);
       __syncwarp();
     }
+    const int rest = count - done;  // below GROUPS
+    int ti = 0, tj = 0;
+    long long ta = 0;
+    if (lane < rest) {
+      ti = qi[warp][done + lane];
+      tj = qj[warp][done + lane];
+      ta = qa[warp][done + lane];
+    }
+    __syncwarp();
+    if (lane < rest) {
+      qi[warp][lane] = ti;
+      qj[warp][lane] = tj;
+      qa[warp][lane] = ta;
+    }
+    count = rest;
+    __syncwarp();
   }
-  if (lane < count) refine_one<H>(a, qi[warp][lane], qj[warp][lane], qa[warp][lane]);
+  if (grp < count) refine_one<H>(a, qi[warp][grp], qj[warp][grp], qa[warp][grp]);
 }
 
 // ---------------- bond 32: one warp per chain ----------------
@@ -708,8 +699,9 @@ DK_API dk_status dk_gram_refine(dk_ctx* ctx, const void* mps_rows, int m_rows, c
       if (ng > 64LL * ctx->sm_count) ng = 64LL * ctx->sm_count;
       rf::norms32_kernel<<<int(ng), rf::WARPS32 * 32, smem32, st>>>(a, n_units);
     } else {
-      long long ng = (n_units + 127) / 128;
-      if (ng > 16LL * ctx->sm_count) ng = 16LL * ctx->sm_count;
+      const int per = 128 / (chi_max == 4 ? rf::LANES<2> : rf::LANES<4>);
+      long long ng = (n_units + per - 1) / per;
+      if (ng > 64LL * ctx->sm_count) ng = 64LL * ctx->sm_count;
       if (chi_max == 4) rf::norms_small_kernel<2><<<int(ng), 128, 0, st>>>(a, n_units);
       else rf::norms_small_kernel<4><<<int(ng), 128, 0, st>>>(a, n_units);
     }
@@ -724,7 +716,8 @@ DK_API dk_status dk_gram_refine(dk_ctx* ctx, const void* mps_rows, int m_rows, c
     rf::refine32_kernel<<<int(grid), rf::WARPS32 * 32, smem, st>>>(a);
     return launch_status();
   }
-  long long grid = (total + rf::SMALL_WARPS * 32 * 8 - 1) / (rf::SMALL_WARPS * 32 * 8);
+  // a warp per 32 entries until the GPU is full: the hits of a small block then run side by side
+  long long grid = (total + rf::SMALL_WARPS * 32 - 1) / (rf::SMALL_WARPS * 32);
   const long long cap = 16LL * ctx->sm_count;
   if (grid > cap) grid = cap;
   if (chi_max == 4) rf::refine_small_kernel<2><<<int(grid), rf::SMALL_WARPS * 32, 0, st>>>(a);

@@ -569,8 +569,202 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
   if (log_norm && live && q == 0) log_norm[i] = chain[0][0].half_log_mod();
 }
 
-// One warp per sample for wide bonds (closed-form block HA >= 4): the same sweep with the
-// matrices in shared memory, lanes parallel over columns and rows.
+// Bonds 8 and 16 (closed-form block HA = 4, 8, stored block HS = HA): one lane per row of M_s,
+// P = 2 HA lanes per (sample, s): two samples a warp at HA = 4, one at 8. Bound by FP64 issue: a warp-wide FP64 instruction holds an SM's FP64 pipe for about 16
+// cycles whether one lane works or all do, so every step is spread over all lanes:
+//  * u_k and w_k of P sites at a time, one sincos per lane, kept in shared memory;
+//  * M_s = R A_s: the bond phases are a Kronecker product of 2 x 2 blocks [[w, w~], [w~, w]] over
+//    the repetitions' bits, so a row of R takes RP - 1 butterflies
+//        (a, b) -> c (a + b) +/- i s (a - b),   w = c + i s,
+//    instead of HA^2 products, and one phase per column;
+//  * Householder QR (the same reflectors and signs as LAPACK's: R_jj = -sigma x_0 / |x_0|) with
+//    dot products over the rows as shuffle sums, roots by rsqrt.
+// Measured, 1000 samples, n = 256, bond 8: 5.1 ms (the warp-per-sample form below: 26.3 ms).
+template <int HA>
+struct WideCfg {
+  static constexpr int P = 2 * HA;                   // rows of M_s = lanes per (sample, s)
+  static constexpr int SAMPLES = 32 / (2 * P);       // per warp
+};
+
+template <int P>
+__device__ __forceinline__ double rows_sum(double v) {
+#pragma unroll
+  for (int o = P / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, P);
+  return v;
+}
+template <int P>
+__device__ __forceinline__ cd rows_sum(cd v) {
+  return mk(rows_sum<P>(v.x), rows_sum<P>(v.y));
+}
+
+template <int HA, int RP>
+__global__ void __launch_bounds__(32) mps_build_rows_kernel(const float* __restrict__ x, int m, int n,
+                                                            double angle_scale, int ent_block, int out_c128,
+                                                            void* __restrict__ out, int32_t* __restrict__ bond) {
+  using Cf = WideCfg<HA>;
+  constexpr int P = Cf::P, CHI = 2 * HA;
+  __shared__ cd fac[Cf::SAMPLES][P][2];                    // u_k, w_k of P sites
+  __shared__ cd Rs[Cf::SAMPLES][2][HA][HA];                // R = diag(R_0, R_1)
+  const int tid = threadIdx.x, smp = tid / (2 * P), in = tid % (2 * P), s = in / P, row = in % P;
+  const int t = row / HA, j0 = row % HA;
+  const int i0 = blockIdx.x * Cf::SAMPLES + smp;
+  const bool live = i0 < m;
+  const int i = live ? i0 : m - 1;  // spare lanes shadow the last sample and store nothing
+  const float* xs = x + size_t(i) * n;
+  for (int e = in; e < 2 * HA * HA; e += 2 * P) (&Rs[smp][0][0][0])[e] = mk(e == 0 ? 1.0 : 0.0, 0.0);
+  int act = 1;
+  for (int k = 0; k < n; ++k) {
+    if (k % P == 0) {
+      __syncwarp();
+      const int kk = k + (in >> 1);
+      if (kk < n) {
+        const double xk = double(xs[kk]);
+        const double arg = (in & 1) == 0 ? -0.5 * angle_scale * xk
+                           : (entangled(ent_block, kk) ? -(PI_D - (kk > 0 ? double(xs[kk - 1]) : 0.0)) * (PI_D - xk)
+                                                       : 0.0);
+        double sn, cs;
+        sincos(arg, &sn, &cs);
+        fac[smp][in >> 1][in & 1] = mk(cs, sn);
+      }
+    }
+    __syncwarp();
+    const cd u = fac[smp][k % P][0], w = fac[smp][k % P][1];
+    const size_t base = (size_t(k) * m + i) * (size_t(CHI) * CHI);
+    if (bond && i0 == 0 && in == 0) bond[k] = act;
+    // this row of M_s: R's row through the bits' butterflies, then the column phases
+    cd b[HA];
+#pragma unroll
+    for (int c = 0; c < HA; ++c) b[c] = Rs[smp][t][j0][c];
+#pragma unroll
+    for (int bit = 1; bit < HA; bit <<= 1)
+#pragma unroll
+      for (int c = 0; c < HA; ++c)
+        if (!(c & bit)) {
+          const cd sum = cadd(b[c], b[c | bit]), dif = csub(b[c], b[c | bit]);
+          const double px = w.x * sum.x, py = w.x * sum.y;
+          b[c] = mk(fma(-w.y, dif.y, px), fma(w.y, dif.x, py));
+          b[c | bit] = mk(fma(w.y, dif.y, px), fma(-w.y, dif.x, py));
+        }
+    {
+      // L(c) of the top bit s times the top bit's bond phase: amp (-1)^popc(c & c >> 1) u^(RP - 2 popc(c)) w^(+-1)
+      constexpr double amp = RP == 3 ? 0.35355339059327376220 : 0.25;
+      cd pw[RP + 1];  // by popc(c): amp w^(+-1) u^(RP - 2 popc(c))
+      const cd wt = mk(amp * w.x, t == s ? amp * w.y : -amp * w.y);
+      cd up = u;      // u^1, u^3, u^5 (RP odd) or u^2, u^4 (RP even), and their conjugates
+      const cd u2 = cmul(u, u);
+      if (RP % 2 == 0) {
+        up = u2;
+        pw[RP / 2] = wt;
+      }
+#pragma unroll
+      for (int e = RP % 2 == 0 ? 2 : 1; e <= RP; e += 2) {
+        pw[(RP - e) / 2] = cmul(wt, up);
+        pw[(RP + e) / 2] = cmul(wt, cconj(up));
+        up = cmul(up, u2);
+      }
+#pragma unroll
+      for (int c = 0; c < HA; ++c) {
+        // popc and sign of the whole index s HA + c
+        const int pc = __popc(c), neg = __popc(c & (c >> 1)) & 1, negt = neg ^ ((c >> (RP - 2)) & 1);
+        const cd f = s ? pw[pc + 1] : pw[pc];
+        const cd v = cmul(f, b[c]);
+        b[c] = (s ? negt : neg) ? mk(-v.x, -v.y) : v;
+      }
+    }
+    if (k == n - 1) {
+      // last site: the row's sum over the block's columns, normalised over both blocks
+      cd v = b[0];
+#pragma unroll
+      for (int c = 1; c < HA; ++c) v = cadd(v, b[c]);
+      double part = rows_sum<P>(cabs2(v));
+      part += __shfl_xor_sync(0xffffffffu, part, P);
+      const double inv = part > 0.0 ? 1.0 / sqrt(part) : 0.0;
+      if (live) {
+        store_cplx(out, base + size_t(s) * HA * CHI + row, cscale(v, inv), out_c128);
+        for (int j = 1; j < HA; ++j) store_cplx(out, base + (size_t(s) * HA + j) * CHI + row, mk(0.0, 0.0), out_c128);
+      }
+      if (bond && i0 == 0 && in == 0) bond[n] = 1;
+      break;
+    }
+    cd(&M)[HA] = b;
+    const int nref = act < HA ? act : HA;
+    double beta[HA];
+    cd my_alpha = mk(0.0, 0.0);  // R's diagonal element of row j0 (rows below HA)
+#pragma unroll
+    for (int j = 0; j < HA; ++j) {
+      double bj = 0.0;
+      if (j < nref) {
+        const cd xj = M[j];
+        const double part = rows_sum<P>(row >= j ? cabs2(xj) : 0.0);
+        const cd x0 = mk(__shfl_sync(0xffffffffu, xj.x, j, P), __shfl_sync(0xffffffffu, xj.y, j, P));
+        cd vj = xj;
+        cd alpha = mk(0.0, 0.0);
+        if (part > 0.0) {
+          const double a2 = cabs2(x0), r0 = a2 > 0.0 ? rsqrt(a2) : 0.0;
+          const double ax0 = a2 * r0, sigma = part * rsqrt(part);
+          const cd ph = a2 > 0.0 ? cscale(x0, r0) : mk(1.0, 0.0);
+          alpha = cscale(ph, -sigma);
+          bj = 1.0 / (sigma * (sigma + ax0));
+          if (row == j) vj = cscale(ph, ax0 + sigma);
+        }
+        if (row == j) {
+          my_alpha = alpha;
+          M[j] = vj;
+        }
+        const cd v = row >= j ? vj : mk(0.0, 0.0);
+#pragma unroll
+        for (int c = 0; c < HA; ++c) {
+          if (c > j) {
+            const cd mc = M[c];
+            const cd wsum = cscale(rows_sum<P>(cconjmul(v, mc)), bj);
+            M[c] = csub(mc, cmul(v, wsum));
+          }
+        }
+      }
+      beta[j] = bj;
+    }
+    __syncwarp();  // everybody has read R
+    // R_s's row j0 from the rows below HA
+    if (t == 0) {
+#pragma unroll
+      for (int c = 0; c < HA; ++c) {
+        cd v = mk(0.0, 0.0);
+        if (j0 < nref) v = c == j0 ? my_alpha : (c > j0 ? M[c] : v);
+        Rs[smp][s][j0][c] = v;
+      }
+    }
+    cd Q[HA];
+    // the explicit Q: the reflectors in reverse order on the first nref unit columns
+#pragma unroll
+    for (int c = 0; c < HA; ++c) Q[c] = mk(row == c && c < nref ? 1.0 : 0.0, 0.0);
+#pragma unroll
+    for (int jj = 0; jj < HA; ++jj) {
+      const int j = HA - 1 - jj;
+      const double bj = beta[j];
+      if (j < nref) {
+        const cd v = row >= j ? M[j] : mk(0.0, 0.0);
+#pragma unroll
+        for (int c = 0; c < HA; ++c) {
+          if (c >= j && c < nref) {
+            const cd qc = Q[c];
+            const cd wsum = cscale(rows_sum<P>(cconjmul(v, qc)), bj);
+            Q[c] = csub(qc, cmul(v, wsum));
+          }
+        }
+      }
+    }
+    if (live) {
+#pragma unroll
+      for (int j = 0; j < HA; ++j) store_cplx(out, base + (size_t(s) * HA + j) * CHI + row, Q[j], out_c128);
+    }
+    act = 2 * nref;
+  }
+}
+
+// Bond 32 (HA = 16): one warp per sample, the matrices in shared memory, lanes parallel over
+// columns and rows. The lane-per-row form above was tried here too (a warp per block s, rows in
+// shared memory): as accurate, but any other rounding of the tensors moves the few pairs whose
+// log K_q the split-BF16 Gram gets worst, so its results were no longer held to what they were.
 template <int HS, int HA>
 struct WarpQr {
   cd R[2][HS][HA];
@@ -719,37 +913,97 @@ __global__ void __launch_bounds__(32) mps_build_warp_kernel(const float* __restr
   }
 }
 
-// ln|<psi~_i|psi~_i>| of the stored tensors, one thread per sample, by the Gram arithmetic.
+// ln|<psi~_i|psi~_i>| of the stored tensors by the Gram arithmetic: 2 H^2 lanes per sample, lane
+// (s, p, c) holding E_s[p][c]. Per site it forms F(t, s, a, c) of transfer.cuh's term() for a = p
+// and both t from row p of E_t (shuffles), then its own E'_s[p][c]: every sum has the operations
+// and the order of term(), so the bits are the Gram diagonal's. A chain is latency bound: one
+// thread per sample took 1.26 ms for 1000 samples at bond 8 and n = 256, a warp each 0.21 ms.
 template <typename real, int H>
-struct GlobalSub {
-  const real* site;  // this sample's compact tensor at the current site
-  __device__ __forceinline__ void operator()(int, int s, int t, Blk<real, H>& blk) const {
-    constexpr int CHI = 2 * H;
+__global__ void __launch_bounds__(128) self_overlap_kernel(const real* __restrict__ mps, int m, int n,
+                                                            float* __restrict__ log_norm) {
+  constexpr int L = 2 * H * H, CHI = 2 * H;
+  constexpr size_t PER = size_t(CHI) * CHI * 2;  // reals per sample-site
+  const int i0 = (blockIdx.x * 128 + threadIdx.x) / L, gl = threadIdx.x % L;
+  const int i = min(i0, m - 1);  // spare groups shadow the last sample
+  const int s = gl / (H * H), p = (gl / H) % H, c = gl % H;
+  const unsigned mask = L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << ((threadIdx.x & 31) & ~(L - 1));
+  real er = gl == 0 ? real(1) : real(0), ei = real(0);
+  int e2 = 0;
+  auto load = [&](int k, int col, real (&vr)[CHI], real (&vi)[CHI]) {  // column `col` of block s
+    const real* a = mps + (size_t(k) * m + i) * PER + size_t(s * H + col) * CHI * 2;
 #pragma unroll
-    for (int j = 0; j < H; ++j)
+    for (int l = 0; l < CHI; ++l) {
+      vr[l] = a[2 * l];
+      vi[l] = a[2 * l + 1];
+    }
+  };
+  real jr[CHI], ji[CHI], ir[CHI], ii[CHI];
+  load(0, c, jr, ji);
+  load(0, p, ir, ii);
+  for (int k = 0; k < n; ++k) {
+    real nr_[CHI], ni_[CHI], mr_[CHI], mi_[CHI];
+    const int kn = min(k + 1, n - 1);  // the next site's tensors arrive under this site's arithmetic
+    load(kn, c, nr_, ni_);
+    load(kn, p, mr_, mi_);
+    real fr[2], fi[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+#pragma unroll
+      for (int b = 0; b < H; ++b) {
+        const int src = (t * H + p) * H + b;
+        const real xr = __shfl_sync(mask, er, src, L), xi = __shfl_sync(mask, ei, src, L);
+        const real ajr = jr[t * H + b], aji = ji[t * H + b];
+        if (b == 0) {
+          fr[t] = xr * ajr;
+          fi[t] = xr * aji;
+        } else {
+          fr[t] = fma(xr, ajr, fr[t]);
+          fi[t] = fma(xr, aji, fi[t]);
+        }
+        fr[t] = fma(-xi, aji, fr[t]);
+        fi[t] = fma(xi, ajr, fi[t]);
+      }
+    }
+    real ar = real(0), aim = real(0);
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
 #pragma unroll
       for (int a = 0; a < H; ++a) {
-        const int idx = 2 * ((s * H + j) * CHI + t * H + a);
-        blk.r[a][j] = site[idx];
-        blk.i[a][j] = site[idx + 1];
+        const int src = (s * H + a) * H + c;
+        const real gr = __shfl_sync(mask, fr[t], src, L), gi = __shfl_sync(mask, fi[t], src, L);
+        const real air = ir[t * H + a], aii = ii[t * H + a];
+        ar = fma(air, gr, ar);
+        aim = fma(air, gi, aim);
+        ar = fma(aii, gi, ar);
+        aim = fma(-aii, gr, aim);
       }
+    er = ar;
+    ei = aim;
+    if (k == n - 1 || (k % RENORM_EVERY) == RENORM_EVERY - 1) {
+      real mx = fmax(real(0), fmax(fabs(er), fabs(ei)));
+#pragma unroll
+      for (int o = L / 2; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(mask, mx, o, L));
+      const int e = RealBits<real>::exponent(mx);
+      const real sc = RealBits<real>::pow2_neg(e);
+      er *= sc;
+      ei *= sc;
+      e2 += e;
+    }
+#pragma unroll
+    for (int l = 0; l < CHI; ++l) {
+      jr[l] = nr_[l];
+      ji[l] = ni_[l];
+      ir[l] = mr_[l];
+      ii[l] = mi_[l];
+    }
   }
-};
-
-template <typename real, int H>
-__global__ void __launch_bounds__(32) self_overlap_kernel(const real* __restrict__ mps, int m, int n,
-                                                           float* __restrict__ log_norm) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  constexpr size_t PER = size_t(2 * H) * (2 * H) * 2;  // reals per sample-site
-  PairE<real, H> st[1][1];
-  st[0][0].init();
-  for (int k = 0; k < n; ++k) {
-    const GlobalSub<real, H> ld{mps + (size_t(k) * m + i) * PER};
-    const bool last = (k == n - 1);
-    site_step<real, H, 1, 1>(st, ld, ld, last || ((k % RENORM_EVERY) == RENORM_EVERY - 1));
-  }
-  log_norm[i] = st[0][0].half_log_mod();
+  PairE<real, H> last;
+  last.b[0].r[0][0] = __shfl_sync(mask, er, 0, L);
+  last.b[0].i[0][0] = __shfl_sync(mask, ei, 0, L);
+  last.b[1].r[0][0] = __shfl_sync(mask, er, H * H, L);
+  last.b[1].i[0][0] = __shfl_sync(mask, ei, H * H, L);
+  last.e2 = e2;
+  if (gl == 0 && i0 < m) log_norm[i0] = last.half_log_mod();
 }
 
 // Threads per CTA of the pair kernel: full warps while there are enough samples to give
@@ -803,14 +1057,18 @@ static dk_status launch_build(const float* x, int m, int n, const dk_fmap* fm, i
     }
     *fused_norm = ln != nullptr;
   } else {
-    const size_t smem = sizeof(WarpQr<HS, HA>);
-    constexpr int RP = HA == 4 ? 3 : HA == 8 ? 4 : 5;
-    auto kern = mps_build_warp_kernel<HS, HA, RP>;
-    if (smem > 48 * 1024) {
+    static_assert(HS == HA, "wide bonds store the closed form's width");
+    if constexpr (HA <= 8) {
+      constexpr int per = WideCfg<HA>::SAMPLES;
+      mps_build_rows_kernel<HA, HA == 4 ? 3 : 4><<<(m + per - 1) / per, 32, 0, st>>>(
+          x, m, n, double(fm->angle_scale), eb, c128, mps, bond);
+    } else {
+      const size_t smem = sizeof(WarpQr<HS, HA>);
+      auto kern = mps_build_warp_kernel<HS, HA, 5>;
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
         return DK_ERR_CUDA;
+      kern<<<m, 32, smem, st>>>(x, m, n, double(fm->angle_scale), eb, c128, mps, bond);
     }
-    kern<<<m, 32, smem, st>>>(x, m, n, double(fm->angle_scale), eb, c128, mps, bond);
   }
   return launch_status();
 }
@@ -863,15 +1121,14 @@ DK_API dk_status dk_mps_build(dk_ctx* ctx, const float* x, int m, int n, const d
 dk_status dk::self_overlap_launch(const void* mps, int m, int n, int chi, dk_dtype dtype, float* log_norm,
                                   cudaStream_t st) {
   using namespace dk;
-  // one warp per CTA: each thread runs a whole n-site chain, so spread the chains over SMs
-  const int grid = (m + 31) / 32;
   if (dtype == DK_C64 && chi == 32) return self_overlap32_launch(mps, m, n, log_norm, st);
+  const int grid = chi == 8 ? (m + 3) / 4 : (m + 15) / 16;  // 128 threads, 32 or 8 a sample
   if (dtype == DK_C64 && chi == 8) {
-    self_overlap_kernel<float, 4><<<grid, 32, 0, st>>>(static_cast<const float*>(mps), m, n, log_norm);
+    self_overlap_kernel<float, 4><<<grid, 128, 0, st>>>(static_cast<const float*>(mps), m, n, log_norm);
   } else if (dtype == DK_C64 && chi == 4) {
-    self_overlap_kernel<float, 2><<<grid, 32, 0, st>>>(static_cast<const float*>(mps), m, n, log_norm);
+    self_overlap_kernel<float, 2><<<grid, 128, 0, st>>>(static_cast<const float*>(mps), m, n, log_norm);
   } else if (dtype == DK_C128 && chi == 4) {
-    self_overlap_kernel<double, 2><<<grid, 32, 0, st>>>(static_cast<const double*>(mps), m, n, log_norm);
+    self_overlap_kernel<double, 2><<<grid, 128, 0, st>>>(static_cast<const double*>(mps), m, n, log_norm);
   } else {
     return DK_ERR_UNSUPPORTED;
   }

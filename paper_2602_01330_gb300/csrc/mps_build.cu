@@ -364,10 +364,19 @@ __device__ __forceinline__ void pi_minus(float v, float& hi, float& lo) {
 // bond-4 chain truncates nothing, so the FP32 sweep only adds rounding of the size of the
 // complex64 storage's own. In FP32 the rotation angles are formed exactly enough by
 // error-free transforms (pi - x and the products as float pairs), so the only FP32 error
-// in a phase is sincosf's. The exponentials of site k+1 are evaluated while site k is factorised;
-// with log_norm set, every thread also runs the Gram's transfer arithmetic on the
-// sample's stored tensors (gathered by shuffles) so that ln|<psi~|psi~>| is bit-identical
-// to the Gram diagonal.
+// in a phase is sincosf's.
+// With log_norm set, the group also runs the Gram's transfer arithmetic on the sample's
+// stored tensors, each thread one element of E with the operations and order of
+// transfer.cuh's term(), so that ln|<psi~|psi~>| is bit-identical to the Gram diagonal.
+//
+// A sample is one dependency chain over the sites, so the kernel is bound by the instructions
+// and latencies of a site: the angles of four sites are evaluated at once, one sincos per
+// thread; of the bond phases w^(2 - 2 popc) of two repetitions only w^2 (same block) or its
+// conjugate (other block) and 1 occur in a thread, likewise u^2 and 1, so a row of M_s takes
+// three complex products; and E advances by site k - 1 beside the Gram-Schmidt sweep of site
+// k, which does not depend on it. 2000 samples at n = 784: 517 us (one sincos per site and
+// thread, phases picked from tables and every thread running all of E: 775 us); 64 samples
+// at n = 8 in complex128: 39 us (108 us).
 template <int HA, int RP, typename real, typename creal>
 __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restrict__ x, int m, int n,
                                                            double angle_scale, int ent_block,
@@ -396,21 +405,21 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
   // -angle_scale / 2 as a float pair (FP32 form)
   const float g_hi = float(-0.5 * angle_scale);
   const float g_lo = float(-0.5 * angle_scale - double(g_hi));
-  // thread q & 1 == 0: u_k = exp(-i angle_scale x_k / 2); q & 1 == 1: w_k =
+  // site k: which = 0: u_k = exp(-i angle_scale x_k / 2); 1: w_k =
   // exp(-i (pi - x_{k-1})(pi - x_k)) (one factor of the RZZ phase, see mps_build_pair_kernel)
-  auto expo = [&](int k) -> C {
+  auto expo = [&](int k, int which) -> C {
     const float xk = xs[k];
     const float xp = k > 0 ? xs[k - 1] : 0.0f;
     const bool ent = entangled(ent_block, k);
     if constexpr (f64) {
-      const double arg = (q & 1) == 0 ? -0.5 * angle_scale * double(xk)
-                                      : (ent ? -(PI_D - double(xp)) * (PI_D - double(xk)) : 0.0);
+      const double arg = which == 0 ? -0.5 * angle_scale * double(xk)
+                                    : (ent ? -(PI_D - double(xp)) * (PI_D - double(xk)) : 0.0);
       double sn, cs;
       sincos(arg, &sn, &cs);
       return mkc(cs, sn);
     } else {
       float hi, lo;
-      if ((q & 1) == 0) {
+      if (which == 0) {
         hi = g_hi * xk;
         lo = fmaf(g_hi, xk, -hi) + g_lo * xk;
       } else if (ent) {
@@ -439,29 +448,102 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
     else return __frsqrt_rn(v);
   };
   constexpr creal TINY = f64 ? creal(1e-300) : creal(1e-30);
-  PairE<real, HS> chain[1][1];
-  chain[0][0].init();
-  C e_cur = expo(0);
-  for (int k = 0; k < n; ++k) {
-    const C e_next = (k + 1 < n) ? expo(k + 1) : mkc(creal(1), creal(0));
-    SiteFactors<RP, creal> f;
-    {
-      const C u = mkc(__shfl_sync(mask, e_cur.x, base_lane), __shfl_sync(mask, e_cur.y, base_lane));
-      const C w = mkc(__shfl_sync(mask, e_cur.x, base_lane + 1), __shfl_sync(mask, e_cur.y, base_lane + 1));
-      f.make_from(u, w);
+
+  // E of the self-overlap: this thread's E_s[t][j] (row t, column j of block s)
+  real er = q == 0 ? real(1) : real(0), ei = real(0);
+  int e2 = 0;
+  // advances E by the site whose stored values are vr, vi in the group's threads
+  auto overlap_step = [&](const real (&vr)[HS], const real (&vi)[HS], bool renorm) {
+    real jr[CHI], ji[CHI], ir[CHI], ii[CHI];  // columns j and t of this block, rows l
+#pragma unroll
+    for (int l = 0; l < CHI; ++l) {
+      const int src = base_lane + 4 * s + l;
+      const real r0 = __shfl_sync(mask, vr[0], src), r1 = __shfl_sync(mask, vr[1], src);
+      const real c0 = __shfl_sync(mask, vi[0], src), c1 = __shfl_sync(mask, vi[1], src);
+      jr[l] = j ? r1 : r0;
+      ji[l] = j ? c1 : c0;
+      ir[l] = t ? r1 : r0;
+      ii[l] = t ? c1 : c0;
     }
+    real fr[2], fi[2];  // F(tt, s, a = t, c = j)
+#pragma unroll
+    for (int tt = 0; tt < 2; ++tt) {
+#pragma unroll
+      for (int b = 0; b < HS; ++b) {
+        const int src = base_lane + 4 * tt + 2 * t + b;
+        const real xr = __shfl_sync(mask, er, src), xi = __shfl_sync(mask, ei, src);
+        const real ajr = jr[tt * HS + b], aji = ji[tt * HS + b];
+        if (b == 0) {
+          fr[tt] = xr * ajr;
+          fi[tt] = xr * aji;
+        } else {
+          fr[tt] = fma(xr, ajr, fr[tt]);
+          fi[tt] = fma(xr, aji, fi[tt]);
+        }
+        fr[tt] = fma(-xi, aji, fr[tt]);
+        fi[tt] = fma(xi, ajr, fi[tt]);
+      }
+    }
+    real ar = real(0), aim = real(0);
+#pragma unroll
+    for (int tt = 0; tt < 2; ++tt)
+#pragma unroll
+      for (int a = 0; a < HS; ++a) {
+        const int src = base_lane + 4 * s + 2 * a + j;
+        const real gr = __shfl_sync(mask, fr[tt], src), gi = __shfl_sync(mask, fi[tt], src);
+        const real air = ir[tt * HS + a], aii = ii[tt * HS + a];
+        ar = fma(air, gr, ar);
+        aim = fma(air, gi, aim);
+        ar = fma(aii, gi, ar);
+        aim = fma(-aii, gr, aim);
+      }
+    er = ar;
+    ei = aim;
+    if (renorm) {
+      real mx = fmax(real(0), fmax(fabs(er), fabs(ei)));
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(mask, mx, o));
+      const int e = RealBits<real>::exponent(mx);
+      const real sc = RealBits<real>::pow2_neg(e);
+      er *= sc;
+      ei *= sc;
+      e2 += e;
+    }
+  };
+  auto rescales = [&](int k) { return k == n - 1 || (k & (RENORM_EVERY - 1)) == RENORM_EVERY - 1; };
+
+  C e_cur = expo(min(q >> 1, n - 1), q & 1);  // the angles of sites 0 .. 3
+  C e_next = e_cur;
+  real pr[HS], pi[HS];  // the stored values of the previous site
+  for (int k = 0; k < n; ++k) {
+    if ((k & 3) == 0) {
+      if (k > 0) e_cur = e_next;
+      if (k + 4 < n) e_next = expo(min(k + 4 + (q >> 1), n - 1), q & 1);
+    }
+    const int sl = base_lane + 2 * (k & 3);
+    const C u = mkc(__shfl_sync(mask, e_cur.x, sl), __shfl_sync(mask, e_cur.y, sl));
+    const C w = mkc(__shfl_sync(mask, e_cur.x, sl + 1), __shfl_sync(mask, e_cur.y, sl + 1));
     if (bond && i0 == 0 && q == 0) bond[k] = act;
+    // this thread's row of M_s = R A_s: closed-form columns c = s HA + cc, left positions t HA + cp
+    C mrow[HA];
+    if constexpr (HA == 1) {
+      constexpr creal amp = creal(0.70710678118654752440);
+      const C acc = cmul(Rrow[0], t == s ? w : cconj(w));
+      mrow[0] = cmul(cscale(s == 0 ? u : cconj(u), amp), acc);
+    } else {
+      const bool same = s == t;
+      const C w2 = cmul(w, w), u2 = cmul(u, u);
+      const C wf = same ? w2 : cconj(w2);
+      const C P = same ? Rrow[0] : Rrow[1], O = same ? Rrow[1] : Rrow[0];
+      const C acc0 = cadd(cmul(P, wf), O), acc1 = cadd(P, cmul(O, wf));
+      const C lu = s == 0 ? cscale(u2, creal(0.5)) : cscale(cconj(u2), creal(-0.5));
+      const C a = cmul(lu, s == 0 ? acc0 : acc1), b = cscale(s == 0 ? acc1 : acc0, creal(0.5));
+      mrow[0] = s == 0 ? a : b;
+      mrow[1] = s == 0 ? b : a;
+    }
+    if (log_norm && k > 0) overlap_step(pr, pi, rescales(k - 1));
     C qv[HS];  // this thread's row of Q_s: stored element (s, jc, l = row) for jc < HS
     if (k < n - 1) {
-      C mrow[HA];
-#pragma unroll
-      for (int cc = 0; cc < HA; ++cc) {
-        const int c = s * HA + cc;
-        C acc = zero;
-#pragma unroll
-        for (int cp = 0; cp < HA; ++cp) acc = cadd(acc, cmul(Rrow[cp], f.bond(t * HA + cp, c)));
-        mrow[cc] = cmul(f.local(c), acc);
-      }
       const int nref = act < HA ? act : HA;
       // classical Gram-Schmidt with one re-orthogonalisation pass over the 4 rows
       C qrow[HA], rcol[HA][HA];
@@ -507,15 +589,8 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
       }
       act = 2 * nref;
     } else {
-      C acc = zero;
-#pragma unroll
-      for (int cc = 0; cc < HA; ++cc) {
-        const int c = s * HA + cc;
-        C inner = zero;
-#pragma unroll
-        for (int cp = 0; cp < HA; ++cp) inner = cadd(inner, cmul(Rrow[cp], f.bond(t * HA + cp, c)));
-        acc = cadd(acc, cmul(f.local(c), inner));
-      }
+      C acc = mrow[0];
+      if constexpr (HA > 1) acc = cadd(mrow[0], mrow[1]);
       creal n2 = cabs2(acc);
       n2 += __shfl_xor_sync(mask, n2, 1);
       n2 += __shfl_xor_sync(mask, n2, 2);
@@ -526,47 +601,31 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
       if (bond && i0 == 0 && q == 0) bond[n] = 1;
     }
     // the stored values, rounded once: to memory and, for the self-overlap, to registers
-    real vr[HS], vi[HS];
 #pragma unroll
     for (int jc = 0; jc < HS; ++jc) {
-      vr[jc] = real(qv[jc].x);
-      vi[jc] = real(qv[jc].y);
+      pr[jc] = real(qv[jc].x);
+      pi[jc] = real(qv[jc].y);
     }
     if (live) {
       const size_t base = (size_t(k) * m + i) * (CHI * CHI);
 #pragma unroll
       for (int jc = 0; jc < HS; ++jc) {
         const size_t idx = base + (s * HS + jc) * CHI + row;
-        if constexpr (c128) reinterpret_cast<double2*>(out)[idx] = make_double2(vr[jc], vi[jc]);
-        else reinterpret_cast<float2*>(out)[idx] = make_float2(vr[jc], vi[jc]);
+        if constexpr (c128) reinterpret_cast<double2*>(out)[idx] = make_double2(pr[jc], pi[jc]);
+        else reinterpret_cast<float2*>(out)[idx] = make_float2(pr[jc], pi[jc]);
       }
     }
-    if (log_norm) {
-      // gather the sample's 16 stored values: element (s', jc, l) from thread 4 s' + l
-      real ar[2][HS][CHI], ai[2][HS][CHI];
-#pragma unroll
-      for (int ss = 0; ss < 2; ++ss)
-#pragma unroll
-        for (int l = 0; l < CHI; ++l)
-#pragma unroll
-          for (int jc = 0; jc < HS; ++jc) {
-            ar[ss][jc][l] = __shfl_sync(mask, vr[jc], base_lane + 4 * ss + l);
-            ai[ss][jc][l] = __shfl_sync(mask, vi[jc], base_lane + 4 * ss + l);
-          }
-      auto ld = [&](int, int ss, int tt, Blk<real, HS>& blk) {
-#pragma unroll
-        for (int jc = 0; jc < HS; ++jc)
-#pragma unroll
-          for (int a = 0; a < HS; ++a) {
-            blk.r[a][jc] = ar[ss][jc][tt * HS + a];
-            blk.i[a][jc] = ai[ss][jc][tt * HS + a];
-          }
-      };
-      site_step<real, HS, 1, 1>(chain, ld, ld, k == n - 1 || ((k & (RENORM_EVERY - 1)) == RENORM_EVERY - 1));
-    }
-    e_cur = e_next;
   }
-  if (log_norm && live && q == 0) log_norm[i] = chain[0][0].half_log_mod();
+  if (log_norm) {
+    overlap_step(pr, pi, true);
+    PairE<real, HS> last;
+    last.b[0].r[0][0] = __shfl_sync(mask, er, base_lane);
+    last.b[0].i[0][0] = __shfl_sync(mask, ei, base_lane);
+    last.b[1].r[0][0] = __shfl_sync(mask, er, base_lane + 4);
+    last.b[1].i[0][0] = __shfl_sync(mask, ei, base_lane + 4);
+    last.e2 = e2;
+    if (live && q == 0) log_norm[i] = last.half_log_mod();
+  }
 }
 
 // Bonds 8 and 16 (closed-form block HA = 4, 8, stored block HS = HA): one lane per row of M_s,

@@ -308,6 +308,149 @@ __global__ void __launch_bounds__(Cfg::NTHREADS, Cfg::MINB)
   }
 }
 
+// Small blocks: 2 H^2 lanes per pair. Lane (s, p, c) holds E_s[p][c] and forms per site the F(t, s,
+// a = p, c) of transfer.cuh's term() for both t from row p of E_t (shuffles), then its own
+// E'_s[p][c]: the operations and order of term(), so the bits are gram_kernel's. A lane's share of
+// a site is 1 / (2 H^2) of the pair's products, but shuffles and operand loads (every lane its
+// own) cost a full GPU several times the tile kernel's time: the better form while the pairs do
+// not fill the GPU and a chain's latency is the launch's. The tensors come straight from global
+// memory, DEPTH sites ahead. K_c's feature sum runs in one lane, in order.
+// Measured against the best tile shape, us: bond 4 FP32, n = 784, symmetric, 40 samples 245
+// (409), 100 samples 350 (413), 150 samples 617 (419); bond 8, n = 256, 40 samples 159 (590), 100
+// samples 458 (650), 150 samples 898 (694); FP64, n = 64, 40 samples 111 (592), 200 samples 770
+// (818), 16 x 2000 rows 1049 (994).
+template <typename real, int H, int DEPTH>
+__global__ void __launch_bounds__(128) gram_lanes_kernel(const real* __restrict__ mps_r, int m_r,
+                                                         const real* __restrict__ mps_c, int m_c, const GramArgs p) {
+  constexpr int L = 2 * H * H, CHI = 2 * H, N4 = CHI * 2 * int(sizeof(real)) / 16;  // 16-byte pieces of a column
+  const long long e = (blockIdx.x * 128LL + threadIdx.x) / L;
+  if (e >= (long long)p.nrows * p.ncols) return;
+  const int rr = int(e / p.ncols), i = p.row0 + rr, j = p.col0 + int(e - (long long)rr * p.ncols);
+  if (p.symmetric && j < i) return;
+  const int gl = threadIdx.x % L, s = gl / (H * H), pp = (gl / H) % H, c = gl % H;
+  const unsigned mask = L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << ((threadIdx.x & 31) & ~(L - 1));
+  // column c of block s of sample j, column pp of block s of sample i: CHI complex numbers each
+  constexpr size_t PER = size_t(CHI) * CHI * 2;
+  const float4* pj = reinterpret_cast<const float4*>(mps_c + size_t(j) * PER + size_t(s * H + c) * CHI * 2);
+  const float4* pi = reinterpret_cast<const float4*>(mps_r + size_t(i) * PER + size_t(s * H + pp) * CHI * 2);
+  const size_t step_j = size_t(m_c) * PER * sizeof(real) / 16, step_i = size_t(m_r) * PER * sizeof(real) / 16;
+  struct Col {
+    float4 v[N4];
+    __device__ __forceinline__ real at(int q) const {  // real number q of the column
+      if constexpr (sizeof(real) == 4) {
+        return f4_get(v[q >> 2], q & 3);
+      } else {
+        const float4 w = v[q >> 1];
+        return (q & 1) ? __hiloint2double(__float_as_int(w.w), __float_as_int(w.z))
+                       : __hiloint2double(__float_as_int(w.y), __float_as_int(w.x));
+      }
+    }
+  };
+  Col bj[DEPTH], bi[DEPTH];
+  auto fetch = [&](int d, int k) {
+    if (k < p.n) {
+#pragma unroll
+      for (int q = 0; q < N4; ++q) {
+        bj[d].v[q] = __ldg(pj + size_t(k) * step_j + q);
+        bi[d].v[q] = __ldg(pi + size_t(k) * step_i + q);
+      }
+    }
+  };
+#pragma unroll
+  for (int d = 0; d < DEPTH; ++d) fetch(d, d);
+  real er = gl == 0 ? real(1) : real(0), ei = real(0);
+  int e2 = 0;
+  for (int k0 = 0; k0 < p.n; k0 += DEPTH) {
+#pragma unroll
+    for (int d = 0; d < DEPTH; ++d) {
+      const int k = k0 + d;
+      if (k < p.n) {
+        const Col vj = bj[d], vi = bi[d];
+        fetch(d, k + DEPTH);
+        real fr[2], fi[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+#pragma unroll
+          for (int b = 0; b < H; ++b) {
+            const int src = (t * H + pp) * H + b;
+            const real xr = __shfl_sync(mask, er, src, L), xi = __shfl_sync(mask, ei, src, L);
+            const real ajr = vj.at(2 * (t * H + b)), aji = vj.at(2 * (t * H + b) + 1);
+            if (b == 0) {
+              fr[t] = xr * ajr;
+              fi[t] = xr * aji;
+            } else {
+              fr[t] = fma(xr, ajr, fr[t]);
+              fi[t] = fma(xr, aji, fi[t]);
+            }
+            fr[t] = fma(-xi, aji, fr[t]);
+            fi[t] = fma(xi, ajr, fi[t]);
+          }
+        }
+        real ar = real(0), aim = real(0);
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+          for (int a = 0; a < H; ++a) {
+            const int src = (s * H + a) * H + c;
+            const real gr = __shfl_sync(mask, fr[t], src, L), gi = __shfl_sync(mask, fi[t], src, L);
+            const real air = vi.at(2 * (t * H + a)), aii = vi.at(2 * (t * H + a) + 1);
+            ar = fma(air, gr, ar);
+            aim = fma(air, gi, aim);
+            ar = fma(aii, gi, ar);
+            aim = fma(-aii, gr, aim);
+          }
+        er = ar;
+        ei = aim;
+        if (k == p.n - 1 || (k & (RENORM_EVERY - 1)) == RENORM_EVERY - 1) {
+          real mx = fmax(real(0), fmax(fabs(er), fabs(ei)));
+#pragma unroll
+          for (int o = L / 2; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(mask, mx, o, L));
+          const int ex = RealBits<real>::exponent(mx);
+          const real sc = RealBits<real>::pow2_neg(ex);
+          er *= sc;
+          ei *= sc;
+          e2 += ex;
+        }
+      }
+    }
+  }
+  PairE<real, H> last;
+  last.b[0].r[0][0] = __shfl_sync(mask, er, 0, L);
+  last.b[0].i[0][0] = __shfl_sync(mask, ei, 0, L);
+  last.b[1].r[0][0] = __shfl_sync(mask, er, H * H, L);
+  last.b[1].i[0][0] = __shfl_sync(mask, ei, H * H, L);
+  last.e2 = e2;
+  if (gl != 0) return;
+  float d2 = 0.0f, comp = 0.0f;
+  if (p.need_kc) {
+    const float* xr = p.x_r + size_t(i) * p.n;
+    const float* xc = p.x_c + size_t(j) * p.n;
+    int f = 0;
+    if ((p.n & 3) == 0 && ((reinterpret_cast<uintptr_t>(p.x_r) | reinterpret_cast<uintptr_t>(p.x_c)) & 15) == 0) {
+#pragma unroll 4
+      for (; f < p.n; f += 4) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(xr + f)), b = __ldg(reinterpret_cast<const float4*>(xc + f));
+        kahan_add_sq(d2, comp, a.x - b.x);
+        kahan_add_sq(d2, comp, a.y - b.y);
+        kahan_add_sq(d2, comp, a.z - b.z);
+        kahan_add_sq(d2, comp, a.w - b.w);
+      }
+    }
+#pragma unroll 4
+    for (; f < p.n; ++f) kahan_add_sq(d2, comp, __ldg(xr + f) - __ldg(xc + f));
+  }
+  write_pair(p, last.half_log_mod(), d2, i, j);
+}
+
+template <typename real, int H, int DEPTH>
+static dk_status launch_lanes(const void* mps_r, int m_r, const void* mps_c, int m_c, const GramArgs& a,
+                              cudaStream_t st) {
+  const long long threads = (long long)a.nrows * a.ncols * (2 * H * H);
+  gram_lanes_kernel<real, H, DEPTH><<<int((threads + 127) / 128), 128, 0, st>>>(
+      static_cast<const real*>(mps_r), m_r, static_cast<const real*>(mps_c), m_c, a);
+  return launch_status();
+}
+
 template <class Cfg>
 struct GramLauncher {
   static dk_status run(dk_ctx* ctx, const void* mps_r, int m_r, const void* mps_c, int m_c, const GramArgs& a,
@@ -362,7 +505,13 @@ using F32_P22tS4 = GramCfg<float, 4, 4, 8, 2, 2, 4, 1, 2, 3, 4>;  // 32 x 16 pai
 using F32_P22qS6 = GramCfg<float, 4, 4, 8, 2, 2, 2, 1, 2, 4, 6>;  // 16 x 16 pairs, 4 CTAs per SM, 6 sites/stage
 using F32_P22vS5 = GramCfg<float, 4, 4, 8, 2, 2, 4, 1, 3, 2, 5>;  // 32 x 16 pairs, 2 CTAs per SM, 3 stages of 5
 using F32_P22oS4 = GramCfg<float, 4, 4, 8, 2, 2, 1, 1, 2, 8, 4>;  // 8 x 16 pairs, one warp, 8 CTAs per SM
-using F64_P11 = GramCfg<double, 4, 4, 8, 1, 1, 4, 2, 4, 1>;    // 16 x 16 pairs, 256 threads
+using F32_P22r2 = GramCfg<float, 4, 1, 32, 2, 2, 1, 1, 2, 8>;     // 2 x 64 pairs, one warp, 8 CTAs per SM
+using F32_P11r1 = GramCfg<float, 4, 1, 32, 1, 1, 1, 1, 3, 16>;    // 1 x 32 pairs, one warp, 16 CTAs per SM
+using F32_P11w = GramCfg<float, 4, 4, 8, 1, 1, 1, 1, 4, 16>;      // 4 x 8 pairs, one warp, 16 CTAs per SM
+// FP64 issues at 2 multiply-adds a cycle and SM, so a tile's time is its pairs and the SMs in
+// use set the rate: one-warp tiles of 32 pairs. 64 samples at n = 8: 77 us, 36 us by the lanes
+// form (16 x 16 tiles with 256 threads: 142 us on 10 SMs).
+using F64_P11 = GramCfg<double, 4, 4, 8, 1, 1, 1, 1, 4, 8>;    // 4 x 8 pairs, one warp, 8 CTAs per SM
 using F32X8_P11 = GramCfg<float, 8, 4, 8, 1, 1, 4, 2, 4, 1>;   // chi = 8: 16 x 16 pairs, 256 threads
 using F32X8_S4 = GramCfg<float, 8, 4, 8, 1, 1, 4, 2, 2, 1, 4>;    // chi = 8: 16 x 16, 2 stages of 4 sites
 using F32X8_S2 = GramCfg<float, 8, 4, 8, 1, 1, 4, 2, 3, 1, 2>;    // chi = 8: 16 x 16, 3 stages of 2 sites
@@ -383,24 +532,78 @@ template <class Cfg>
 constexpr CfgInfo info_of() {
   return CfgInfo{Cfg::TR, Cfg::TC, Cfg::NTHREADS};
 }
-// Shapes selectable for complex64 / chi 4, in id order 1..19; the built-in choice is kF32Chi4Default.
+// Shapes selectable for complex64 / chi 4, in id order 1..22; the built-in choice is f32_shape's.
 static const CfgInfo kF32Chi4[] = {info_of<F32_P11>(),  info_of<F32_P21>(),  info_of<F32_P22>(), info_of<F32_P12>(),
                                    info_of<F32_P22w>(), info_of<F32_P21w>(), info_of<F32_P14>(),
                                    info_of<F32_P22wS2>(), info_of<F32_P22S2>(), info_of<F32_P22wS4>(),
                                    info_of<F32_P22wS8>(), info_of<F32_P22S8>(),
                                    info_of<F32_P22hS8>(), info_of<F32_P22vS8>(), info_of<F32_P22qS4>(),
                                    info_of<F32_P22tS4>(), info_of<F32_P22qS6>(), info_of<F32_P22vS5>(),
-                                   info_of<F32_P22oS4>()};
-constexpr int kF32Chi4Default = 17;  // 16 x 16 pairs, 4 CTAs per SM, 6-site stages: fastest on the n = 784 Gram and rows
+                                   info_of<F32_P22oS4>(), info_of<F32_P22r2>(), info_of<F32_P11r1>(),
+                                   info_of<F32_P11w>()};
+constexpr int kF32Chi4Default = 17;  // 16 x 16 pairs, 4 CTAs per SM, 6-site stages: fastest where tiles fill many waves
+
+// The built-in complex64 / chi 4 shape for a block: the least estimated time over a few shapes,
+// from what a site costs a wave of CTAs in ns, measured at n = 784 against 8000 columns: `full`
+// a full wave, `low` one with at most per_low CTAs per SM (a warp per scheduler; for shape 17
+// two CTAs often share two schedulers), equal steps of per_low CTAs in between. Few rows leave
+// most of a 16-row tile empty, and a wave of four-pair threads takes the chain's latency however
+// few CTAs it has, so small blocks take narrower tiles and one pair per thread. Measured, us,
+// against shape 17: 8000 columns at n = 784 with 1 row 446 (1126), 5 rows 725 (1127), 37 rows
+// 2546 (3272), 100 rows 6430 (6613); symmetric 40 samples 417 (614). Where shape 17 needs 8
+// waves or more its last one matters little and it is taken at once.
+struct ShapeCost {
+  int id, tile_rows, tile_cols, per_sm, per_low, steps;
+  float full, low;
+};
+static const ShapeCost kF32Shapes[] = {{17, 16, 16, 4, 1, 1, 1439.0f, 785.0f},
+                                       {19, 8, 16, 8, 4, 1, 1490.0f, 927.0f},
+                                       {20, 2, 64, 8, 4, 1, 1630.0f, 1050.0f},
+                                       {21, 1, 32, 16, 4, 3, 1600.0f, 560.0f},
+                                       {22, 4, 8, 16, 4, 3, 1130.0f, 600.0f}};
+
+static int f32_shape(const dk_ctx* ctx, const GramArgs& a) {
+  int best = kF32Chi4Default;
+  float best_t = 0.0f;
+  for (const ShapeCost& c : kF32Shapes) {
+    GramArgs t = a;
+    const long long tiles = count_tiles(t, c.tile_rows, c.tile_cols);
+    const long long slots = (long long)ctx->sm_count * c.per_sm, waves = tiles / slots, rest = tiles % slots;
+    if (c.id == kF32Chi4Default && waves >= 8) return c.id;
+    float time = float(waves) * c.full;
+    if (rest > 0) {
+      const int k = int((rest + ctx->sm_count - 1) / ctx->sm_count), step = (k - 1) / c.per_low;
+      time += c.low + float(step < c.steps ? step : c.steps) / float(c.steps) * (c.full - c.low);
+    }
+    // within 4 % the tail of a long launch decides less than the estimate says: shape 17
+    if (c.id == kF32Chi4Default || time < best_t) {
+      best = c.id;
+      best_t = c.id == kF32Chi4Default ? 0.96f * time : time;
+    }
+  }
+  return best;
+}
 static const CfgInfo kF64Chi4[] = {info_of<F64_P11>()};
 constexpr int kF32Chi8Default = 2;  // 16 x 16 pairs, 2 stages of 4 sites: fastest at d = 256
 static const CfgInfo kF32Chi8[] = {info_of<F32X8_P11>(), info_of<F32X8_S4>(), info_of<F32X8_S2>(),
                                    info_of<F32X8_h>(), info_of<F32X8_q>()};
 
+// Pairs per SM up to which gram_lanes_kernel takes a block: between the sizes measured there (the
+// bond-4 and bond-8 FP32 forms only where no tile shape is set).
+constexpr long long kLanesF32Chi4 = 40, kLanesF64Chi4 = 150, kLanesF32Chi8 = 50;
+
+// Pairs a block computes.
+static long long pair_count(const GramArgs& a) {
+  const long long n = (long long)a.nrows * a.ncols;
+  return a.symmetric ? (n + a.nrows) / 2 : n;
+}
+
 static dk_status gram_dispatch(dk_ctx* ctx, const void* mps_r, int m_r, const void* mps_c, int m_c, int chi,
                                dk_dtype dtype, dk_precision prec, const GramArgs& a, cudaStream_t st) {
   if (dtype == DK_C64 && prec == DK_PREC_F32 && chi == 4) {
-    const int id = ctx->gram_config > 0 ? ctx->gram_config : kF32Chi4Default;
+    if (ctx->gram_config == 0 && pair_count(a) <= kLanesF32Chi4 * ctx->sm_count)
+      return launch_lanes<float, 2, 4>(mps_r, m_r, mps_c, m_c, a, st);
+    const int id = ctx->gram_config > 0 ? ctx->gram_config : f32_shape(ctx, a);
     switch (id) {
       case 1: return launch_gram<F32_P11>(ctx, mps_r, m_r, mps_c, m_c, a, st);
       case 2: return launch_gram<F32_P21>(ctx, mps_r, m_r, mps_c, m_c, a, st);
@@ -420,13 +623,20 @@ static dk_status gram_dispatch(dk_ctx* ctx, const void* mps_r, int m_r, const vo
       case 17: return launch_gram<F32_P22qS6>(ctx, mps_r, m_r, mps_c, m_c, a, st);
       case 18: return launch_gram<F32_P22vS5>(ctx, mps_r, m_r, mps_c, m_c, a, st);
       case 19: return launch_gram<F32_P22oS4>(ctx, mps_r, m_r, mps_c, m_c, a, st);
+      case 20: return launch_gram<F32_P22r2>(ctx, mps_r, m_r, mps_c, m_c, a, st);
+      case 21: return launch_gram<F32_P11r1>(ctx, mps_r, m_r, mps_c, m_c, a, st);
+      case 22: return launch_gram<F32_P11w>(ctx, mps_r, m_r, mps_c, m_c, a, st);
       case 3: return launch_gram<F32_P22>(ctx, mps_r, m_r, mps_c, m_c, a, st);
       default: return launch_gram<F32_P22qS6>(ctx, mps_r, m_r, mps_c, m_c, a, st);
     }
   }
+  if (dtype == DK_C128 && prec == DK_PREC_F64 && chi == 4 && pair_count(a) <= kLanesF64Chi4 * ctx->sm_count)
+    return launch_lanes<double, 2, 2>(mps_r, m_r, mps_c, m_c, a, st);
   if (dtype == DK_C128 && prec == DK_PREC_F64 && chi == 4)
     return launch_gram<F64_P11>(ctx, mps_r, m_r, mps_c, m_c, a, st);
   if (dtype == DK_C64 && prec == DK_PREC_F32 && chi == 8) {
+    if (ctx->gram_config == 0 && pair_count(a) <= kLanesF32Chi8 * ctx->sm_count)
+      return launch_lanes<float, 4, 2>(mps_r, m_r, mps_c, m_c, a, st);
     // shape ids index the bond-8 table; an id beyond it (e.g. one chosen for bond 4) gives
     // the default
     switch (ctx->gram_config) {

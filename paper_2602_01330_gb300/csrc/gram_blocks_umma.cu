@@ -23,10 +23,12 @@
 //             Im of row r, adds log2 |G_B|^2 to its running sums and frees the accumulator
 //             (narrow: two accumulators, so block B's epilogue runs under the MMAs of block
 //             B + 1); after an item's last block it writes the tile through the common
-//             epilogue (write_pair) with the squared distances of the RBF kernel, which
-//             rbf_d2_kernel computed beforehand (feature rows staged through shared memory,
-//             the per-pair Kahan FP32 sum of every Gram kernel), or, when a rectangular
-//             tile's blocks are split over several items, its partial log2 sums.
+//             epilogue (write_pair) with the squared distances of the RBF kernel, or, when a
+//             rectangular tile's blocks are split over several items, its partial log2 sums;
+//   warps 10-11 (RBF form) the tile's squared distances for K_c, on the CUDA cores that the
+//             MMAs leave idle: 64 x 32 pairs at a time, feature rows staged through shared
+//             memory, the per-pair Kahan FP32 sum of every Gram kernel. Without these warps
+//             rbf_d2_kernel computes the distances beforehand.
 //
 // Self-norms (diagonal mode): a unit is one (diagonal tile, block) pair with A = B in shared
 // memory. The diagonal tile of the symmetric Gram issues the same instructions on the same
@@ -49,6 +51,18 @@ constexpr int BM = 128;     // tile rows = MMA M = TMEM lanes
 constexpr int ROWB = 128;   // one 16-amplitude chunk of a sample: 4 planes x 16 BF16
 constexpr int NEPI = 8;     // epilogue warps
 constexpr int NTHREADS = (2 + NEPI) * 32;
+// Warps of the RBF form: two is what the register file holds beside the epilogue's 168
+// registers a thread. They are hidden where the MMAs of a tile take longer: a block of b
+// qubits costs 2^b / 16 chunks of 0.47 us for its b features, 1.7 us a feature at b = 9, 0.94 at
+// b = 8, where the distances take 1280 FP32 operations a lane, 0.7 us at the least. The line is
+// drawn at b = 9. 2000 samples of 780 features, K only: 1.49 ms against 1.83 ms with
+// rbf_d2_kernel before it (b = 9), 2.35 against 2.70 ms (b = 10); one tile (100 samples, where
+// rbf_d2_kernel is short): 1.45 against 1.58 ms and 2.29 against 2.43 ms.
+constexpr int NRBF = 2;
+constexpr int RBF_F = 16;            // features staged at a time
+constexpr int RBF_R = 64, RBF_C = 32;  // pairs of a pass: 8 x 4 per thread
+constexpr size_t RBF_SMEM = size_t(RBF_F) * (RBF_R + RBF_C) * sizeof(float);
+constexpr int RBF_MIN_CPB = 32;
 
 // BN columns per tile. Narrow form (WIDE = false): N = BN instructions into [Re | Im]
 // accumulators, two of them (double-buffered). Wide form (BN = 128): the column rows are
@@ -139,11 +153,11 @@ __device__ __forceinline__ float abs2(float re, float im) { return fmaf(re, re, 
 // log2 sums go to part[split][i - row0][j - col0] for split_finish_kernel. Diagonal mode
 // (diag = 1): n_units = ceil(m_diag / 128) * nb items (diagonal tile, block) over the states
 // of tm_r, |G_B(i, i)|^2 written to g2_out[blk][i].
-template <int BN, bool WIDE>
-__global__ void __launch_bounds__(NTHREADS, 1)
+template <int BN, bool WIDE, bool RBF>
+__global__ void __launch_bounds__(NTHREADS + (RBF ? NRBF * 32 : 0), 1)
     gram_blocks_umma_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_constant__ CUtensorMap tm_c,
                             const GramArgs p, int nb, int cpb, int diag, int n_units, float* __restrict__ g2_out,
-                            int m_diag, int ksplit, float* __restrict__ part) {
+                            int m_diag, int ksplit, float* __restrict__ part, float* d2_out) {
   using C = Cfg<BN, WIDE>;
   constexpr int NSTAGES = C::NST;
   extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -155,6 +169,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t* done = acc_empty + 2;
   u32* tmem_slot = reinterpret_cast<u32*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* d2_items = abort_flag + 1;  // items of this CTA whose distances are written
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -168,6 +183,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
     mbar_init(done, 1);
     *abort_flag = 0;
+    *d2_items = 0;
     fence_mbar_init();
     prefetch_tensormap(&tm_r);
     if (!diag) prefetch_tensormap(&tm_c);
@@ -310,6 +326,70 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       tc_commit(done);
       if (!mbar_wait_bounded(done, 0u)) record_status(p.status, DEV_TIMEOUT);
     }
+  } else if (RBF && warp >= 2 + NEPI) {
+    // ---- squared distances of the items' pairs ----
+    float* xr = reinterpret_cast<float*>(smem + NSTAGES * C::STAGE + 256);  // [feature][row]
+    float* xc = xr + RBF_F * RBF_R;                                        // [feature][column]
+    const int rt = tid - NTHREADS, ty = rt >> 3, tx = rt & 7;  // rows 8 ty .. + 7, columns 4 tx .. + 3
+    int done = 0;
+    // no look at the abort flag: these two warps meet at barrier 1 and have nothing to wait for
+    for (int w = bid; w < n_items; w += grid) {
+      int r0, c0, b0, b1, split;
+      item(w, r0, c0, b0, b1, split);
+      for (int sub = 0; sub < (BM / RBF_R) * (BN / RBF_C); ++sub) {
+        const int pr0 = r0 + (sub % (BM / RBF_R)) * RBF_R, pc0 = c0 + (sub / (BM / RBF_R)) * RBF_C;
+        // nothing of the pass in the block, or (symmetric) all of it below the diagonal
+        if (pr0 >= p.row0 + p.nrows || pc0 >= p.col0 + p.ncols || (p.symmetric && pc0 + RBF_C - 1 < pr0)) continue;
+        float s[8][4], cmp[8][4];
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) s[a][b] = cmp[a][b] = 0.0f;
+        // thread rt stages row pr0 + rt and, with the lanes of half a warp, half of column pc0 + rt / 2
+        const float* gr = p.x_r + size_t(min(pr0 + rt, p.row0 + p.nrows - 1)) * p.n;
+        const float* gc = p.x_c + size_t(min(pc0 + (rt >> 1), p.col0 + p.ncols - 1)) * p.n;
+        const int h = (rt & 1) * (RBF_F / 2);
+        for (int f0 = 0; f0 < p.n; f0 += RBF_F) {
+          const int nf = min(RBF_F, p.n - f0);
+          float vr[RBF_F], vc[RBF_F / 2];
+#pragma unroll
+          for (int f = 0; f < RBF_F; ++f) vr[f] = f < nf ? __ldg(gr + f0 + f) : 0.0f;
+#pragma unroll
+          for (int f = 0; f < RBF_F / 2; ++f) vc[f] = h + f < nf ? __ldg(gc + f0 + h + f) : 0.0f;
+          asm volatile("bar.sync 1, 64;" ::: "memory");  // the previous chunk has been read
+#pragma unroll
+          for (int f = 0; f < RBF_F; ++f) xr[f * RBF_R + rt] = vr[f];
+#pragma unroll
+          for (int f = 0; f < RBF_F / 2; ++f) xc[(h + f) * RBF_C + (rt >> 1)] = vc[f];
+          asm volatile("bar.sync 1, 64;" ::: "memory");
+#pragma unroll 1
+          for (int f = 0; f < nf; ++f) {
+            const float4 ra = *reinterpret_cast<const float4*>(xr + f * RBF_R + 8 * ty);
+            const float4 rb = *reinterpret_cast<const float4*>(xr + f * RBF_R + 8 * ty + 4);
+            const float4 cb = *reinterpret_cast<const float4*>(xc + f * RBF_C + 4 * tx);
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+              for (int b = 0; b < 4; ++b)
+                kahan_add_sq(s[a][b], cmp[a][b], (a < 4 ? f4_get(ra, a) : f4_get(rb, a - 4)) - f4_get(cb, b));
+          }
+        }
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const int i = pr0 + 8 * ty + a, j = pc0 + 4 * tx + b;
+            if (i < p.row0 + p.nrows && j < p.col0 + p.ncols)
+              d2_out[size_t(i - p.row0) * size_t(p.ncols) + size_t(j - p.col0)] = s[a][b];
+          }
+      }
+      __threadfence_block();
+      asm volatile("bar.sync 1, 64;" ::: "memory");
+      if (rt == 0) {
+        __threadfence_block();
+        *d2_items = ++done;
+      }
+    }
   } else {
     // ---- epilogue ----
     const int q = warp & 3;           // the TMEM lane quarter this warp may access
@@ -320,8 +400,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
     for (int u = 0; u < C::CPT; ++u) lg[u] = 0.0f;
     long long k = 0;
+    int n_done = 0;  // items finished before this one
     bool stop = false;
-    for (int w = bid; w < n_items && !stop; w += grid) {
+    for (int w = bid; w < n_items && !stop; w += grid, ++n_done) {
       int r0, c0, b0, b1, split;
       item(w, r0, c0, b0, b1, split);
       const int i = r0 + r;
@@ -367,6 +448,24 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
       }
       if (diag || stop) continue;
+      if (RBF) {
+        // the item's distances: usually there long before (bounded)
+        unsigned long long t0 = 0;
+        while (*d2_items <= n_done) {
+          const unsigned long long now = globaltimer_ns();
+          if (t0 == 0) t0 = now;
+          if (now - t0 > WAIT_LIMIT_NS || *abort_flag) {
+            stop = true;
+            break;
+          }
+        }
+        __threadfence_block();
+        if (__any_sync(0xffffffffu, stop)) {
+          if (lane == 0) give_up();
+          stop = true;
+          break;
+        }
+      }
       // end of the item: the tile's outputs, or (split over the blocks) its partial log sums
 #pragma unroll
       for (int u = 0; u < C::CPT; ++u) {
@@ -376,7 +475,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (ksplit > 1) {
           if (valid) part[size_t(split) * size_t(p.nrows) * size_t(p.ncols) + at] = lg[u];
         } else {
-          write_pair(p, half_log_lg(lg[u]), (valid && p.need_kc) ? p.d2[at] : 0.0f, i, j);
+          write_pair(p, half_log_lg(lg[u]), (valid && p.need_kc) ? (RBF ? d2_out : p.d2)[at] : 0.0f, i, j);
         }
         lg[u] = 0.0f;
       }
@@ -480,10 +579,14 @@ dk_status encode_states_map(dk_ctx* ctx, CUtensorMap* map, const void* states, i
 
 // The shared-memory opt-in is a per-device, per-function attribute: it is set before every
 // launch (a cheap host call), so no process-wide flag has to track devices or threads.
-template <int BN, bool WIDE>
+template <int BN, bool WIDE, bool RBF>
+constexpr size_t smem_of() {
+  return Cfg<BN, WIDE>::SMEM + (RBF ? RBF_SMEM : 0);
+}
+template <int BN, bool WIDE, bool RBF = false>
 dk_status set_smem() {
-  if (cudaFuncSetAttribute(gram_blocks_umma_kernel<BN, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(Cfg<BN, WIDE>::SMEM)) != cudaSuccess)
+  if (cudaFuncSetAttribute(gram_blocks_umma_kernel<BN, WIDE, RBF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           int(smem_of<BN, WIDE, RBF>())) != cudaSuccess)
     return DK_ERR_CUDA;
   return DK_OK;
 }
@@ -511,16 +614,18 @@ dk_status launch_gram(dk_ctx* ctx, const void* sr, int m_r, const void* sc, int 
   CUtensorMap tr, tc;
   dk_status s = encode_states_map(ctx, &tr, sr, m_r, nb, dp, BM);
   if (s == DK_OK) s = encode_states_map(ctx, &tc, sc, m_c, nb, dp, BN);
-  if (s == DK_OK) s = set_smem<BN, WIDE>();
+  // distances beside the MMAs where the item's blocks take long enough to hide them
+  const bool rbf = WIDE && a.need_kc && ksplit == 1 && dp / 16 >= RBF_MIN_CPB;
+  if (s == DK_OK) s = rbf ? set_smem<BN, WIDE, WIDE>() : set_smem<BN, WIDE>();
   if (s != DK_OK) return s;
   a.ntiles = count_tiles(a, BM, BN);  // also sets the tile grid (tiles_r, tiles_c) the kernel decodes
   if (a.ntiles != ntiles) return DK_ERR_ARG;
   const long long items = (long long)ntiles * ksplit;
   const int grid = int(items < ctx->sm_count ? items : ctx->sm_count);
   if (grid < 1) return DK_OK;
-  // squared distances of the RBF kernel first, into the caller's scratch
+  // otherwise the squared distances of the RBF kernel first; both into the caller's scratch
   float* d2 = need.d2_bytes ? static_cast<float*>(ws) : nullptr;
-  if (a.need_kc) {
+  if (a.need_kc && !rbf) {
     GramArgs ar = a;
     ar.ntiles = count_tiles(ar, RT, RT);
     const int rgrid = ar.ntiles < 8 * ctx->sm_count ? ar.ntiles : 8 * ctx->sm_count;
@@ -531,8 +636,12 @@ dk_status launch_gram(dk_ctx* ctx, const void* sr, int m_r, const void* sc, int 
   float* part = need.part_bytes ? reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + need.d2_bytes) : nullptr;
   const size_t np = size_t(a.nrows) * size_t(a.ncols);
   if (s == DK_OK) {
-    gram_blocks_umma_kernel<BN, WIDE><<<grid, NTHREADS, Cfg<BN, WIDE>::SMEM, st>>>(tr, tc, a, nb, dp / 16, 0, 0,
-                                                                                   nullptr, 0, ksplit, part);
+    if (rbf)
+      gram_blocks_umma_kernel<BN, WIDE, WIDE><<<grid, NTHREADS + NRBF * 32, smem_of<BN, WIDE, WIDE>(), st>>>(
+          tr, tc, a, nb, dp / 16, 0, 0, nullptr, 0, ksplit, part, d2);
+    else
+      gram_blocks_umma_kernel<BN, WIDE, false><<<grid, NTHREADS, smem_of<BN, WIDE, false>(), st>>>(
+          tr, tc, a, nb, dp / 16, 0, 0, nullptr, 0, ksplit, part, nullptr);
     s = launch_status();
   }
   if (s == DK_OK && part) {
@@ -601,8 +710,8 @@ dk_status block_selfnorm_umma_launch(dk_ctx* ctx, const void* states, int m, int
   GramArgs a{};
   a.status = ctx->status;
   const int grid = int(units < ctx->sm_count ? units : ctx->sm_count);
-  gram_blocks_umma_kernel<128, true><<<grid, NTHREADS, Cfg<128, true>::SMEM, st>>>(t, t, a, nb, dp / 16, 1, int(units),
-                                                                                  g2, m, 1, nullptr);
+  gram_blocks_umma_kernel<128, true, false><<<grid, NTHREADS, smem_of<128, true, false>(), st>>>(
+      t, t, a, nb, dp / 16, 1, int(units), g2, m, 1, nullptr, nullptr);
   s = launch_status();
   if (s == DK_OK) {
     selfnorm_sum_kernel<<<(m + 255) / 256, 256, 0, st>>>(g2, m, nb, log_norm);

@@ -67,16 +67,22 @@ __device__ __forceinline__ float half_log_lg(float lg) { return lg * (0.5f * 0.6
 // The operand form of the tensor-core Grams, same 8 bytes per amplitude as complex64: per
 // chunk of 16 amplitudes one 128-byte row of four BF16 planes [hi_re | hi_im | lo_re | lo_im]
 // of 16 values each, v ~ hi + lo; zeros past the dim amplitudes of the state.
+// Two amplitudes per thread and step: 4-byte stores.
 __device__ inline void store_split(float2* out, const float2* psf, int dim, int dp) {
-  __nv_bfloat16* pl = reinterpret_cast<__nv_bfloat16*>(out);
-  for (int k = threadIdx.x; k < dp; k += BUILD_NT) {
-    const float vr = k < dim ? psf[k].x : 0.0f, vi = k < dim ? psf[k].y : 0.0f;
-    const __nv_bfloat16 hr = __float2bfloat16_rn(vr), hi = __float2bfloat16_rn(vi);
-    __nv_bfloat16* row = pl + (k >> 4) * 64 + (k & 15);
-    row[0] = hr;
-    row[16] = hi;
-    row[32] = __float2bfloat16_rn(vr - __bfloat162float(hr));
-    row[48] = __float2bfloat16_rn(vi - __bfloat162float(hi));
+  uint32_t* pl = reinterpret_cast<uint32_t*>(out);
+  for (int k = 2 * threadIdx.x; k < dp; k += 2 * BUILD_NT) {
+    const float4 v = k < dim ? *reinterpret_cast<const float4*>(psf + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float wx = k + 1 < dim ? v.z : 0.0f, wy = k + 1 < dim ? v.w : 0.0f;  // dim = 1: one amplitude
+    auto pack = [](__nv_bfloat16 a, __nv_bfloat16 b) {
+      return uint32_t(__bfloat16_as_ushort(a)) | (uint32_t(__bfloat16_as_ushort(b)) << 16);
+    };
+    const __nv_bfloat16 r0 = __float2bfloat16_rn(v.x), i0 = __float2bfloat16_rn(v.y);
+    const __nv_bfloat16 r1 = __float2bfloat16_rn(wx), i1 = __float2bfloat16_rn(wy);
+    uint32_t* row = pl + (k >> 4) * 32 + ((k & 15) >> 1);
+    row[0] = pack(r0, r1);
+    row[8] = pack(i0, i1);
+    row[16] = pack(__float2bfloat16_rn(v.x - __bfloat162float(r0)), __float2bfloat16_rn(wx - __bfloat162float(r1)));
+    row[24] = pack(__float2bfloat16_rn(v.y - __bfloat162float(i0)), __float2bfloat16_rn(wy - __bfloat162float(i1)));
   }
 }
 

@@ -35,6 +35,8 @@
 // Gram diagonal exactly 1.
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 #include "transfer.cuh"
@@ -369,16 +371,35 @@ __device__ __forceinline__ void pi_minus(float v, float& hi, float& lo) {
 // stored tensors, each thread one element of E with the operations and order of
 // transfer.cuh's term(), so that ln|<psi~|psi~>| is bit-identical to the Gram diagonal.
 //
-// A sample is one dependency chain over the sites, so the kernel is bound by the instructions
-// and latencies of a site: the angles of four sites are evaluated at once, one sincos per
-// thread; of the bond phases w^(2 - 2 popc) of two repetitions only w^2 (same block) or its
-// conjugate (other block) and 1 occur in a thread, likewise u^2 and 1, so a row of M_s takes
-// three complex products; and E advances by site k - 1 beside the Gram-Schmidt sweep of site
-// k, which does not depend on it. 2000 samples at n = 784: 517 us (one sincos per site and
-// thread, phases picked from tables and every thread running all of E: 775 us); 64 samples
-// at n = 8 in complex128: 39 us (108 us).
+// A sample is one dependency chain over the sites (the Gram-Schmidt sweep and R), so the kernel
+// is bound by that chain's latency and by whatever one warp has to issue beside it. Three warps
+// share a sample's work, OCT_CH sites at a time through two shared-memory buffers each way:
+//   warp 1  the angles of the coming sites, one sincos per lane;
+//   warp 0  the chain: of the bond phases w^(2 - 2 popc) of two repetitions only w^2 (same
+//           block) or its conjugate (other block) and 1 occur in a thread, likewise u^2 and 1,
+//           so a row of M_s takes three complex products;
+//   warp 2  (with log_norm) E of the self-overlap from the stored values.
+// They meet at named barriers, each a warp that arrives and a warp that waits; the waits end
+// because every role runs over the same chunks in the same order. Idle lanes (fewer than four
+// samples a CTA) repeat the last sample and store nothing.
+// 2000 samples at n = 784: 396 us (all roles in one warp: 517 us); 37 samples: 367 us
+// (498 us); 64 samples at n = 8 in complex128: 38 us (39 us).
+constexpr int OCT_CH = 8;
+// named barriers: one of each kind per buffer (immediate ids, so that a CTA reserves 9 of them)
+enum { OCT_ANG_FULL = 1, OCT_ANG_FREE = 3, OCT_Q_FULL = 5, OCT_Q_FREE = 7 };
+template <int ID>
+__device__ __forceinline__ void pair_sync(int buffer) {
+  if (buffer) asm volatile("bar.sync %0, 64;" ::"n"(ID + 1) : "memory");
+  else asm volatile("bar.sync %0, 64;" ::"n"(ID) : "memory");
+}
+template <int ID>
+__device__ __forceinline__ void pair_arrive(int buffer) {
+  if (buffer) asm volatile("bar.arrive %0, 64;" ::"n"(ID + 1) : "memory");
+  else asm volatile("bar.arrive %0, 64;" ::"n"(ID) : "memory");
+}
+
 template <int HA, int RP, typename real, typename creal>
-__global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restrict__ x, int m, int n,
+__global__ void __launch_bounds__(96) mps_build_oct_kernel(const float* __restrict__ x, int m, int n, int spc,
                                                            double angle_scale, int ent_block,
                                                            void* __restrict__ out, int32_t* __restrict__ bond,
                                                            float* __restrict__ log_norm) {
@@ -386,22 +407,22 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
   constexpr int HS = 2, CHI = 4;
   constexpr bool c128 = sizeof(real) == 8;   // stored precision
   constexpr bool f64 = sizeof(creal) == 8;   // arithmetic precision
+  const int warp = threadIdx.x >> 5, grp = (threadIdx.x >> 3) & 3;  // grp: sample of the CTA
   const int q = threadIdx.x & 7;
   const int s = q >> 2, t = (q >> 1) & 1, j = q & 1;
   const int row = t * HS + j;  // this thread's left-bond position
-  const int i0 = blockIdx.x * (blockDim.x >> 3) + (threadIdx.x >> 3);
-  const unsigned mask = blockDim.x >= 32 ? 0xffffffffu : ((1u << blockDim.x) - 1u);
-  const bool live = i0 < m;
-  const int i = live ? i0 : m - 1;
-  const int base_lane = threadIdx.x & ~7;
+  const int i0 = blockIdx.x * spc + grp;
+  constexpr unsigned mask = 0xffffffffu;
+  const bool live = grp < spc && i0 < m;
+  const int i = i0 < m ? i0 : m - 1;
+  const int base_lane = threadIdx.x & 24;
+  const int nch = (n + OCT_CH - 1) / OCT_CH;
   const float* xs = x + size_t(i) * n;
   const C zero = mkc(creal(0), creal(0));
-  // Rrow[cp] = R_t[j][cp]: row j of the previous site's block-t factor (HA columns)
-  C Rrow[HA];
-#pragma unroll
-  for (int c = 0; c < HA; ++c) Rrow[c] = zero;
-  if (t == 0 && j == 0) Rrow[0] = mkc(creal(1), creal(0));
-  int act = 1;
+  // [buffer][site][sample]: u, w (HA = 2: u^2, w^2); the stored values in their stored order
+  constexpr int QS = HS * HS * CHI * 2 + 16 / int(sizeof(real));
+  __shared__ __align__(16) creal ang[2][OCT_CH][4][4];
+  __shared__ __align__(16) real qs[2][OCT_CH][4][QS];
   // -angle_scale / 2 as a float pair (FP32 form)
   const float g_hi = float(-0.5 * angle_scale);
   const float g_lo = float(-0.5 * angle_scale - double(g_hi));
@@ -437,10 +458,113 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
       return expi_split(hi, lo);
     }
   };
-  auto gsum = [&](creal v) {  // sum over the 4 threads of this block
-    v += __shfl_xor_sync(mask, v, 1);
-    v += __shfl_xor_sync(mask, v, 2);
-    return v;
+  if (warp == 1) {
+    for (int c = 0; c < nch; ++c) {
+      if (c >= 2) pair_sync<OCT_ANG_FREE>(c & 1);
+#pragma unroll
+      for (int r = 0; r < OCT_CH / 4; ++r) {
+        const int o = 4 * r + (q >> 1);
+        C v = expo(min(c * OCT_CH + o, n - 1), q & 1);
+        if constexpr (HA == 2) v = cmul(v, v);
+        ang[c & 1][o][grp][2 * (q & 1)] = v.x;
+        ang[c & 1][o][grp][2 * (q & 1) + 1] = v.y;
+      }
+      pair_arrive<OCT_ANG_FULL>(c & 1);
+    }
+    return;
+  }
+  auto rescales = [&](int k) { return k == n - 1 || (k & (RENORM_EVERY - 1)) == RENORM_EVERY - 1; };
+  if (warp == 2) {
+    // E of the self-overlap: this thread's E_s[t][j] (row t, column j of block s)
+    real er = q == 0 ? real(1) : real(0), ei = real(0);
+    int e2 = 0;
+    for (int k = 0; k < n; ++k) {
+      const int ch = k / OCT_CH, h = ch & 1;
+      if (k % OCT_CH == 0) {
+        if (k > 0 && ch + 1 < nch) pair_arrive<OCT_Q_FREE>(h ^ 1);  // chunk ch - 1, for ch + 1
+        pair_sync<OCT_Q_FULL>(h);
+      }
+      // columns j and t of this block, rows l
+      real cj[2 * CHI], ct[2 * CHI];
+      const real* col = qs[h][k % OCT_CH][grp] + s * HS * CHI * 2;
+      using V = typename std::conditional<c128, double2, float4>::type;
+      constexpr int PER = 16 / int(sizeof(real));
+#pragma unroll
+      for (int l = 0; l < 2 * CHI / PER; ++l) {
+        *reinterpret_cast<V*>(cj + l * PER) = reinterpret_cast<const V*>(col + j * CHI * 2)[l];
+        *reinterpret_cast<V*>(ct + l * PER) = reinterpret_cast<const V*>(col + t * CHI * 2)[l];
+      }
+      real fr[2], fi[2];  // F(tt, s, a = t, c = j)
+#pragma unroll
+      for (int tt = 0; tt < 2; ++tt) {
+#pragma unroll
+        for (int b = 0; b < HS; ++b) {
+          const int src = base_lane + 4 * tt + 2 * t + b;
+          const real xr = __shfl_sync(mask, er, src), xi = __shfl_sync(mask, ei, src);
+          const real ajr = cj[2 * (tt * HS + b)], aji = cj[2 * (tt * HS + b) + 1];
+          if (b == 0) {
+            fr[tt] = xr * ajr;
+            fi[tt] = xr * aji;
+          } else {
+            fr[tt] = fma(xr, ajr, fr[tt]);
+            fi[tt] = fma(xr, aji, fi[tt]);
+          }
+          fr[tt] = fma(-xi, aji, fr[tt]);
+          fi[tt] = fma(xi, ajr, fi[tt]);
+        }
+      }
+      real ar = real(0), aim = real(0);
+#pragma unroll
+      for (int tt = 0; tt < 2; ++tt)
+#pragma unroll
+        for (int a = 0; a < HS; ++a) {
+          const int src = base_lane + 4 * s + 2 * a + j;
+          const real gr = __shfl_sync(mask, fr[tt], src), gi = __shfl_sync(mask, fi[tt], src);
+          const real air = ct[2 * (tt * HS + a)], aii = ct[2 * (tt * HS + a) + 1];
+          ar = fma(air, gr, ar);
+          aim = fma(air, gi, aim);
+          ar = fma(aii, gi, ar);
+          aim = fma(-aii, gr, aim);
+        }
+      er = ar;
+      ei = aim;
+      if (rescales(k)) {
+        real mx = fmax(real(0), fmax(fabs(er), fabs(ei)));
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(mask, mx, o));
+        const int e = RealBits<real>::exponent(mx);
+        const real sc = RealBits<real>::pow2_neg(e);
+        er *= sc;
+        ei *= sc;
+        e2 += e;
+      }
+    }
+    PairE<real, HS> last;
+    last.b[0].r[0][0] = __shfl_sync(mask, er, base_lane);
+    last.b[0].i[0][0] = __shfl_sync(mask, ei, base_lane);
+    last.b[1].r[0][0] = __shfl_sync(mask, er, base_lane + 4);
+    last.b[1].i[0][0] = __shfl_sync(mask, ei, base_lane + 4);
+    last.e2 = e2;
+    if (live && q == 0) log_norm[i] = last.half_log_mod();
+    return;
+  }
+  // Rrow[cp] = R_t[j][cp]: row j of the previous site's block-t factor (HA columns)
+  C Rrow[HA];
+#pragma unroll
+  for (int c = 0; c < HA; ++c) Rrow[c] = zero;
+  if (t == 0 && j == 0) Rrow[0] = mkc(creal(1), creal(0));
+  int act = 1;
+  // sum over the 4 threads of this block: (v + v^1) + (v^2 + v^3), in FP32 with the three
+  // shuffles in flight together, in FP64 in the two additions of a butterfly
+  auto gsum = [&](creal v) {
+    if constexpr (f64) {
+      v += __shfl_xor_sync(mask, v, 1);
+      v += __shfl_xor_sync(mask, v, 2);
+      return v;
+    } else {
+      const creal a = __shfl_xor_sync(mask, v, 1), b = __shfl_xor_sync(mask, v, 2), c = __shfl_xor_sync(mask, v, 3);
+      return (v + a) + (b + c);
+    }
   };
   auto gsumc = [&](C v) { return mkc(gsum(v.x), gsum(v.y)); };
   auto inv_sqrt = [](creal v) -> creal {
@@ -449,80 +573,18 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
   };
   constexpr creal TINY = f64 ? creal(1e-300) : creal(1e-30);
 
-  // E of the self-overlap: this thread's E_s[t][j] (row t, column j of block s)
-  real er = q == 0 ? real(1) : real(0), ei = real(0);
-  int e2 = 0;
-  // advances E by the site whose stored values are vr, vi in the group's threads
-  auto overlap_step = [&](const real (&vr)[HS], const real (&vi)[HS], bool renorm) {
-    real jr[CHI], ji[CHI], ir[CHI], ii[CHI];  // columns j and t of this block, rows l
-#pragma unroll
-    for (int l = 0; l < CHI; ++l) {
-      const int src = base_lane + 4 * s + l;
-      const real r0 = __shfl_sync(mask, vr[0], src), r1 = __shfl_sync(mask, vr[1], src);
-      const real c0 = __shfl_sync(mask, vi[0], src), c1 = __shfl_sync(mask, vi[1], src);
-      jr[l] = j ? r1 : r0;
-      ji[l] = j ? c1 : c0;
-      ir[l] = t ? r1 : r0;
-      ii[l] = t ? c1 : c0;
-    }
-    real fr[2], fi[2];  // F(tt, s, a = t, c = j)
-#pragma unroll
-    for (int tt = 0; tt < 2; ++tt) {
-#pragma unroll
-      for (int b = 0; b < HS; ++b) {
-        const int src = base_lane + 4 * tt + 2 * t + b;
-        const real xr = __shfl_sync(mask, er, src), xi = __shfl_sync(mask, ei, src);
-        const real ajr = jr[tt * HS + b], aji = ji[tt * HS + b];
-        if (b == 0) {
-          fr[tt] = xr * ajr;
-          fi[tt] = xr * aji;
-        } else {
-          fr[tt] = fma(xr, ajr, fr[tt]);
-          fi[tt] = fma(xr, aji, fi[tt]);
-        }
-        fr[tt] = fma(-xi, aji, fr[tt]);
-        fi[tt] = fma(xi, ajr, fi[tt]);
-      }
-    }
-    real ar = real(0), aim = real(0);
-#pragma unroll
-    for (int tt = 0; tt < 2; ++tt)
-#pragma unroll
-      for (int a = 0; a < HS; ++a) {
-        const int src = base_lane + 4 * s + 2 * a + j;
-        const real gr = __shfl_sync(mask, fr[tt], src), gi = __shfl_sync(mask, fi[tt], src);
-        const real air = ir[tt * HS + a], aii = ii[tt * HS + a];
-        ar = fma(air, gr, ar);
-        aim = fma(air, gi, aim);
-        ar = fma(aii, gi, ar);
-        aim = fma(-aii, gr, aim);
-      }
-    er = ar;
-    ei = aim;
-    if (renorm) {
-      real mx = fmax(real(0), fmax(fabs(er), fabs(ei)));
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(mask, mx, o));
-      const int e = RealBits<real>::exponent(mx);
-      const real sc = RealBits<real>::pow2_neg(e);
-      er *= sc;
-      ei *= sc;
-      e2 += e;
-    }
-  };
-  auto rescales = [&](int k) { return k == n - 1 || (k & (RENORM_EVERY - 1)) == RENORM_EVERY - 1; };
-
-  C e_cur = expo(min(q >> 1, n - 1), q & 1);  // the angles of sites 0 .. 3
-  C e_next = e_cur;
-  real pr[HS], pi[HS];  // the stored values of the previous site
   for (int k = 0; k < n; ++k) {
-    if ((k & 3) == 0) {
-      if (k > 0) e_cur = e_next;
-      if (k + 4 < n) e_next = expo(min(k + 4 + (q >> 1), n - 1), q & 1);
+    const int ch = k / OCT_CH, h = ch & 1;
+    if (k % OCT_CH == 0) {
+      if (k > 0 && ch + 1 < nch) pair_arrive<OCT_ANG_FREE>(h ^ 1);  // chunk ch - 1, for ch + 1
+      pair_sync<OCT_ANG_FULL>(h);
+      if (log_norm) {
+        if (k > 0) pair_arrive<OCT_Q_FULL>(h ^ 1);
+        if (ch >= 2) pair_sync<OCT_Q_FREE>(h);
+      }
     }
-    const int sl = base_lane + 2 * (k & 3);
-    const C u = mkc(__shfl_sync(mask, e_cur.x, sl), __shfl_sync(mask, e_cur.y, sl));
-    const C w = mkc(__shfl_sync(mask, e_cur.x, sl + 1), __shfl_sync(mask, e_cur.y, sl + 1));
+    const creal* uw = ang[h][k % OCT_CH][grp];
+    const C u = mkc(uw[0], uw[1]), w = mkc(uw[2], uw[3]);  // HA = 2: u^2, w^2
     if (bond && i0 == 0 && q == 0) bond[k] = act;
     // this thread's row of M_s = R A_s: closed-form columns c = s HA + cc, left positions t HA + cp
     C mrow[HA];
@@ -532,16 +594,14 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
       mrow[0] = cmul(cscale(s == 0 ? u : cconj(u), amp), acc);
     } else {
       const bool same = s == t;
-      const C w2 = cmul(w, w), u2 = cmul(u, u);
-      const C wf = same ? w2 : cconj(w2);
+      const C wf = same ? w : cconj(w);
       const C P = same ? Rrow[0] : Rrow[1], O = same ? Rrow[1] : Rrow[0];
       const C acc0 = cadd(cmul(P, wf), O), acc1 = cadd(P, cmul(O, wf));
-      const C lu = s == 0 ? cscale(u2, creal(0.5)) : cscale(cconj(u2), creal(-0.5));
+      const C lu = s == 0 ? cscale(u, creal(0.5)) : cscale(cconj(u), creal(-0.5));
       const C a = cmul(lu, s == 0 ? acc0 : acc1), b = cscale(s == 0 ? acc1 : acc0, creal(0.5));
       mrow[0] = s == 0 ? a : b;
       mrow[1] = s == 0 ? b : a;
     }
-    if (log_norm && k > 0) overlap_step(pr, pi, rescales(k - 1));
     C qv[HS];  // this thread's row of Q_s: stored element (s, jc, l = row) for jc < HS
     if (k < n - 1) {
       const int nref = act < HA ? act : HA;
@@ -600,32 +660,22 @@ __global__ void __launch_bounds__(32) mps_build_oct_kernel(const float* __restri
       qv[1] = zero;
       if (bond && i0 == 0 && q == 0) bond[n] = 1;
     }
-    // the stored values, rounded once: to memory and, for the self-overlap, to registers
+    // the stored values, rounded once: to memory and, for the self-overlap, to warp 2
+    const size_t base = (size_t(k) * m + i) * (CHI * CHI);
 #pragma unroll
     for (int jc = 0; jc < HS; ++jc) {
-      pr[jc] = real(qv[jc].x);
-      pi[jc] = real(qv[jc].y);
-    }
-    if (live) {
-      const size_t base = (size_t(k) * m + i) * (CHI * CHI);
-#pragma unroll
-      for (int jc = 0; jc < HS; ++jc) {
-        const size_t idx = base + (s * HS + jc) * CHI + row;
-        if constexpr (c128) reinterpret_cast<double2*>(out)[idx] = make_double2(pr[jc], pi[jc]);
-        else reinterpret_cast<float2*>(out)[idx] = make_float2(pr[jc], pi[jc]);
+      const int at = (s * HS + jc) * CHI + row;
+      const real vr = real(qv[jc].x), vi = real(qv[jc].y);
+      if constexpr (c128) {
+        if (live) reinterpret_cast<double2*>(out)[base + at] = make_double2(vr, vi);
+        if (log_norm) reinterpret_cast<double2*>(qs[h][k % OCT_CH][grp])[at] = make_double2(vr, vi);
+      } else {
+        if (live) reinterpret_cast<float2*>(out)[base + at] = make_float2(vr, vi);
+        if (log_norm) reinterpret_cast<float2*>(qs[h][k % OCT_CH][grp])[at] = make_float2(vr, vi);
       }
     }
   }
-  if (log_norm) {
-    overlap_step(pr, pi, true);
-    PairE<real, HS> last;
-    last.b[0].r[0][0] = __shfl_sync(mask, er, base_lane);
-    last.b[0].i[0][0] = __shfl_sync(mask, ei, base_lane);
-    last.b[1].r[0][0] = __shfl_sync(mask, er, base_lane + 4);
-    last.b[1].i[0][0] = __shfl_sync(mask, ei, base_lane + 4);
-    last.e2 = e2;
-    if (live && q == 0) log_norm[i] = last.half_log_mod();
-  }
+  if (log_norm) pair_arrive<OCT_Q_FULL>(((nch - 1) & 1));
 }
 
 // Bonds 8 and 16 (closed-form block HA = 4, 8, stored block HS = HA): one lane per row of M_s,
@@ -1095,12 +1145,13 @@ static dk_status launch_build(const float* x, int m, int n, const dk_fmap* fm, i
       const int spc = (m + 3) / 4 >= sm_count ? 4 : ((m + 1) / 2 >= sm_count ? 2 : 1);
       const int grid = (m + spc - 1) / spc;
       const double as = double(fm->angle_scale);
+      const int nt = ln ? 96 : 64;
       if (c128) {
-        mps_build_oct_kernel<HA, RP, double, double><<<grid, 8 * spc, 0, st>>>(x, m, n, as, eb, mps, bond, ln);
+        mps_build_oct_kernel<HA, RP, double, double><<<grid, nt, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
       } else if (fp64_qr) {
-        mps_build_oct_kernel<HA, RP, float, double><<<grid, 8 * spc, 0, st>>>(x, m, n, as, eb, mps, bond, ln);
+        mps_build_oct_kernel<HA, RP, float, double><<<grid, nt, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
       } else {
-        mps_build_oct_kernel<HA, RP, float, float><<<grid, 8 * spc, 0, st>>>(x, m, n, as, eb, mps, bond, ln);
+        mps_build_oct_kernel<HA, RP, float, float><<<grid, nt, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
       }
       *fused_norm = ln != nullptr;
       return launch_status();

@@ -378,12 +378,13 @@ __device__ __forceinline__ void pi_minus(float v, float& hi, float& lo) {
 //   warp 0  the chain: of the bond phases w^(2 - 2 popc) of two repetitions only w^2 (same
 //           block) or its conjugate (other block) and 1 occur in a thread, likewise u^2 and 1,
 //           so a row of M_s takes three complex products;
-//   warp 2  (with log_norm) E of the self-overlap from the stored values.
+//   warp 2  writes the tensors out and, with log_norm, advances E of the self-overlap.
 // They meet at named barriers, each a warp that arrives and a warp that waits; the waits end
 // because every role runs over the same chunks in the same order. Idle lanes (fewer than four
 // samples a CTA) repeat the last sample and store nothing.
-// 2000 samples at n = 784: 396 us (all roles in one warp: 517 us); 37 samples: 367 us
-// (498 us); 64 samples at n = 8 in complex128: 38 us (39 us).
+// 2000 samples at n = 784: 289 us (all roles in one warp: 517 us; tensors stored by warp 0, the
+// first site's short bond tested at every site and __frsqrt_rn: 396 us); 37 samples: 253 us
+// (498 us); 64 samples at n = 8 in complex128: 37 us (39 us).
 constexpr int OCT_CH = 8;
 // named barriers: one of each kind per buffer (immediate ids, so that a CTA reserves 9 of them)
 enum { OCT_ANG_FULL = 1, OCT_ANG_FREE = 3, OCT_Q_FULL = 5, OCT_Q_FREE = 7 };
@@ -475,7 +476,7 @@ __global__ void __launch_bounds__(96) mps_build_oct_kernel(const float* __restri
   }
   auto rescales = [&](int k) { return k == n - 1 || (k & (RENORM_EVERY - 1)) == RENORM_EVERY - 1; };
   if (warp == 2) {
-    // E of the self-overlap: this thread's E_s[t][j] (row t, column j of block s)
+    // stores the tensors; E of the self-overlap: this thread's E_s[t][j] (row t, column j of block s)
     real er = q == 0 ? real(1) : real(0), ei = real(0);
     int e2 = 0;
     for (int k = 0; k < n; ++k) {
@@ -484,11 +485,19 @@ __global__ void __launch_bounds__(96) mps_build_oct_kernel(const float* __restri
         if (k > 0 && ch + 1 < nch) pair_arrive<OCT_Q_FREE>(h ^ 1);  // chunk ch - 1, for ch + 1
         pair_sync<OCT_Q_FULL>(h);
       }
-      // columns j and t of this block, rows l
-      real cj[2 * CHI], ct[2 * CHI];
-      const real* col = qs[h][k % OCT_CH][grp] + s * HS * CHI * 2;
       using V = typename std::conditional<c128, double2, float4>::type;
       constexpr int PER = 16 / int(sizeof(real));
+      // the sample's tensor to memory: 32 reals, a 16-byte piece or two per thread
+      const real* site = qs[h][k % OCT_CH][grp];
+      if (live) {
+        V* dst = reinterpret_cast<V*>(static_cast<real*>(out) + (size_t(k) * m + i) * (CHI * CHI * 2));
+#pragma unroll
+        for (int e = 0; e < 4 / PER; ++e) dst[8 * e + q] = reinterpret_cast<const V*>(site)[8 * e + q];
+      }
+      if (!log_norm) continue;
+      // columns j and t of this block, rows l
+      real cj[2 * CHI], ct[2 * CHI];
+      const real* col = site + s * HS * CHI * 2;
 #pragma unroll
       for (int l = 0; l < 2 * CHI / PER; ++l) {
         *reinterpret_cast<V*>(cj + l * PER) = reinterpret_cast<const V*>(col + j * CHI * 2)[l];
@@ -539,6 +548,7 @@ __global__ void __launch_bounds__(96) mps_build_oct_kernel(const float* __restri
         e2 += e;
       }
     }
+    if (!log_norm) return;
     PairE<real, HS> last;
     last.b[0].r[0][0] = __shfl_sync(mask, er, base_lane);
     last.b[0].i[0][0] = __shfl_sync(mask, ei, base_lane);
@@ -569,19 +579,18 @@ __global__ void __launch_bounds__(96) mps_build_oct_kernel(const float* __restri
   auto gsumc = [&](C v) { return mkc(gsum(v.x), gsum(v.y)); };
   auto inv_sqrt = [](creal v) -> creal {
     if constexpr (f64) return rsqrt(v);
-    else return __frsqrt_rn(v);
+    else return rsqrt_chain(v);
   };
   constexpr creal TINY = f64 ? creal(1e-300) : creal(1e-30);
 
-  for (int k = 0; k < n; ++k) {
+  auto build_site = [&](int k, auto first) {
+    constexpr int nref = decltype(first)::value ? 1 : HA;  // columns of Q: the bond is full from site 1 on
     const int ch = k / OCT_CH, h = ch & 1;
     if (k % OCT_CH == 0) {
       if (k > 0 && ch + 1 < nch) pair_arrive<OCT_ANG_FREE>(h ^ 1);  // chunk ch - 1, for ch + 1
       pair_sync<OCT_ANG_FULL>(h);
-      if (log_norm) {
-        if (k > 0) pair_arrive<OCT_Q_FULL>(h ^ 1);
-        if (ch >= 2) pair_sync<OCT_Q_FREE>(h);
-      }
+      if (k > 0) pair_arrive<OCT_Q_FULL>(h ^ 1);
+      if (ch >= 2) pair_sync<OCT_Q_FREE>(h);
     }
     const creal* uw = ang[h][k % OCT_CH][grp];
     const C u = mkc(uw[0], uw[1]), w = mkc(uw[2], uw[3]);  // HA = 2: u^2, w^2
@@ -604,7 +613,6 @@ __global__ void __launch_bounds__(96) mps_build_oct_kernel(const float* __restri
     }
     C qv[HS];  // this thread's row of Q_s: stored element (s, jc, l = row) for jc < HS
     if (k < n - 1) {
-      const int nref = act < HA ? act : HA;
       // classical Gram-Schmidt with one re-orthogonalisation pass over the 4 rows
       C qrow[HA], rcol[HA][HA];
 #pragma unroll
@@ -655,27 +663,25 @@ __global__ void __launch_bounds__(96) mps_build_oct_kernel(const float* __restri
       n2 += __shfl_xor_sync(mask, n2, 1);
       n2 += __shfl_xor_sync(mask, n2, 2);
       n2 += __shfl_xor_sync(mask, n2, 4);
-      const creal inv = n2 > creal(0) ? inv_sqrt(n2) : creal(0);
+      creal inv = creal(0);
+      if constexpr (f64) inv = n2 > creal(0) ? rsqrt(n2) : creal(0);
+      else inv = n2 > creal(0) ? __frsqrt_rn(n2) : creal(0);
       qv[0] = cscale(acc, inv);
       qv[1] = zero;
       if (bond && i0 == 0 && q == 0) bond[n] = 1;
     }
-    // the stored values, rounded once: to memory and, for the self-overlap, to warp 2
-    const size_t base = (size_t(k) * m + i) * (CHI * CHI);
+    // the stored values, rounded once, to warp 2
 #pragma unroll
     for (int jc = 0; jc < HS; ++jc) {
       const int at = (s * HS + jc) * CHI + row;
       const real vr = real(qv[jc].x), vi = real(qv[jc].y);
-      if constexpr (c128) {
-        if (live) reinterpret_cast<double2*>(out)[base + at] = make_double2(vr, vi);
-        if (log_norm) reinterpret_cast<double2*>(qs[h][k % OCT_CH][grp])[at] = make_double2(vr, vi);
-      } else {
-        if (live) reinterpret_cast<float2*>(out)[base + at] = make_float2(vr, vi);
-        if (log_norm) reinterpret_cast<float2*>(qs[h][k % OCT_CH][grp])[at] = make_float2(vr, vi);
-      }
+      if constexpr (c128) reinterpret_cast<double2*>(qs[h][k % OCT_CH][grp])[at] = make_double2(vr, vi);
+      else reinterpret_cast<float2*>(qs[h][k % OCT_CH][grp])[at] = make_float2(vr, vi);
     }
-  }
-  if (log_norm) pair_arrive<OCT_Q_FULL>(((nch - 1) & 1));
+  };
+  build_site(0, std::true_type{});
+  for (int k = 1; k < n; ++k) build_site(k, std::false_type{});
+  pair_arrive<OCT_Q_FULL>((nch - 1) & 1);
 }
 
 // Bonds 8 and 16 (closed-form block HA = 4, 8, stored block HS = HA): one lane per row of M_s,
@@ -1145,13 +1151,12 @@ static dk_status launch_build(const float* x, int m, int n, const dk_fmap* fm, i
       const int spc = (m + 3) / 4 >= sm_count ? 4 : ((m + 1) / 2 >= sm_count ? 2 : 1);
       const int grid = (m + spc - 1) / spc;
       const double as = double(fm->angle_scale);
-      const int nt = ln ? 96 : 64;
       if (c128) {
-        mps_build_oct_kernel<HA, RP, double, double><<<grid, nt, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
+        mps_build_oct_kernel<HA, RP, double, double><<<grid, 96, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
       } else if (fp64_qr) {
-        mps_build_oct_kernel<HA, RP, float, double><<<grid, nt, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
+        mps_build_oct_kernel<HA, RP, float, double><<<grid, 96, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
       } else {
-        mps_build_oct_kernel<HA, RP, float, float><<<grid, nt, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
+        mps_build_oct_kernel<HA, RP, float, float><<<grid, 96, 0, st>>>(x, m, n, spc, as, eb, mps, bond, ln);
       }
       *fused_norm = ln != nullptr;
       return launch_status();

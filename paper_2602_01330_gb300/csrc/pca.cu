@@ -117,7 +117,7 @@ __device__ __forceinline__ float4 pair_rotation(float aii, float ajj, float aij)
     // angle that zeroes a_ij: tau = (a_jj - a_ii) / (2 a_ij), t the smaller root
     const float tau = (ajj - aii) / (2.0f * aij);
     t = (tau >= 0.0f ? 1.0f : -1.0f) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
-    c = __frsqrt_rn(1.0f + t * t);  // correctly rounded: c^2 + s^2 - 1 stays unbiased
+    c = rsqrt_chain(1.0f + t * t);  // correctly rounded: c^2 + s^2 - 1 stays unbiased
     s = t * c;
   }
   return make_float4(c, s, t, 0.0f);

@@ -33,62 +33,95 @@ namespace pca {
 
 constexpr int T32 = 32;
 
-__global__ void __launch_bounds__(256) col_stats_kernel(const float* __restrict__ x, int m, int p,
-                                                        float* __restrict__ mean, float* __restrict__ scale) {
-  const int c = blockIdx.x * 32 + (threadIdx.x & 31), rg = threadIdx.x >> 5;
-  __shared__ double red[8][32];
-  __shared__ double s_mean[32];
+// 8 columns x 8 row groups per CTA (two warps): FP64 issue bounds it, one warp instruction per 16
+// cycles and SM, so the columns are spread over many SMs. 2000 x 784: 68 us (32 columns per CTA,
+// eight warps on each of 25 SMs: 100 us). Every sum keeps its order.
+__global__ void __launch_bounds__(64) col_stats_kernel(const float* __restrict__ x, int m, int p,
+                                                       float* __restrict__ mean, float* __restrict__ scale) {
+  constexpr int NC = 8;
+  const int lc = threadIdx.x & (NC - 1), c = blockIdx.x * NC + lc, rg = threadIdx.x / NC;
+  __shared__ double red[8][NC];
+  __shared__ double s_mean[NC];
   double s = 0.0;
-  if (c < p)
+  if (c < p) {
+#pragma unroll 8
     for (int r = rg; r < m; r += 8) s += double(x[(long long)r * p + c]);
-  red[rg][threadIdx.x & 31] = s;
+  }
+  red[rg][lc] = s;
   __syncthreads();
   if (rg == 0) {
     double t = 0.0;
-    for (int g = 0; g < 8; ++g) t += red[g][threadIdx.x];
-    s_mean[threadIdx.x] = t / m;
+    for (int g = 0; g < 8; ++g) t += red[g][lc];
+    s_mean[lc] = t / m;
   }
   __syncthreads();
-  const double mu = s_mean[threadIdx.x & 31];
+  const double mu = s_mean[lc];
   double q = 0.0;
-  if (c < p)
+  if (c < p) {
+#pragma unroll 8
     for (int r = rg; r < m; r += 8) {
       const double d = double(x[(long long)r * p + c]) - mu;
       q += d * d;
     }
+  }
   __syncthreads();
-  red[rg][threadIdx.x & 31] = q;
+  red[rg][lc] = q;
   __syncthreads();
   if (rg == 0 && c < p) {
     double t = 0.0;
-    for (int g = 0; g < 8; ++g) t += red[g][threadIdx.x];
+    for (int g = 0; g < 8; ++g) t += red[g][lc];
     const double var = t / m;
     mean[c] = float(mu);
     scale[c] = var > 0.0 ? float(sqrt(var)) : 1.0f;
   }
 }
 
-// C[i][j] = sum_r z_ri z_rj / (m - 1), z_rc = (x_rc - mean_c) / scale_c; 32 x 32 tiles
+// C[i][j] = sum_r z_ri z_rj / (m - 1), z_rc = (x_rc - mean_c) / scale_c: 32 x 32 tiles on and
+// above the diagonal, written to both sides (a product's factors commute, so the two sums are the
+// same); the next 32 rows are loaded under the products of these. Bound by the loads' latency and
+// the divisions. 2000 x 784: 172 us (every tile, loads and products in turn: 255 us).
 __global__ void __launch_bounds__(256) cov_kernel(const float* __restrict__ x, int m, int p,
                                                   const float* __restrict__ mean, const float* __restrict__ scale,
                                                   float* __restrict__ A) {
-  __shared__ float zi[T32][T32 + 1], zj[T32][T32 + 1];
-  const int i0 = blockIdx.y * T32, j0 = blockIdx.x * T32;
+  __shared__ __align__(16) float zi[T32][T32], zj[T32][T32];
+  // tile row ti holds the tiles (ti, ti) .. (ti, nt - 1)
+  const int nt = (p + T32 - 1) / T32;
+  int ti = 0, tj = blockIdx.x;
+  while (tj >= nt - ti) tj -= nt - ti++;
+  const int i0 = ti * T32, j0 = (ti + tj) * T32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 rows of 4 outputs per thread
+  // this thread stages columns i0 + tx and j0 + tx of rows ty, ty + 8, ty + 16, ty + 24
+  const int ci = i0 + tx, cj = j0 + tx;
+  const float mi = ci < p ? mean[ci] : 0.0f, si = ci < p ? scale[ci] : 1.0f;
+  const float mj = cj < p ? mean[cj] : 0.0f, sj = cj < p ? scale[cj] : 1.0f;
+  float vi[4], vj[4];
+  auto load = [&](int r0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = r0 + ty + 8 * q;
+      vi[q] = r < m && ci < p ? x[(long long)r * p + ci] : mi;
+      vj[q] = r < m && cj < p ? x[(long long)r * p + cj] : mj;
+    }
+  };
   float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  load(0);
   for (int r0 = 0; r0 < m; r0 += T32) {
-    for (int e = threadIdx.x; e < T32 * T32; e += 256) {
-      const int rr = e / T32, cc = e % T32, r = r0 + rr;
-      const int ci = i0 + cc, cj = j0 + cc;
-      zi[rr][cc] = (r < m && ci < p) ? (x[(long long)r * p + ci] - mean[ci]) / scale[ci] : 0.0f;
-      zj[rr][cc] = (r < m && cj < p) ? (x[(long long)r * p + cj] - mean[cj]) / scale[cj] : 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      // beyond the data the loads gave the mean itself: a zero
+      zi[ty + 8 * q][tx] = r0 + ty + 8 * q < m ? (vi[q] - mi) / si : 0.0f;
+      zj[ty + 8 * q][tx] = r0 + ty + 8 * q < m ? (vj[q] - mj) / sj : 0.0f;
     }
     __syncthreads();
+    if (r0 + T32 < m) load(r0 + T32);
 #pragma unroll 8
     for (int rr = 0; rr < T32; ++rr) {
       const float b = zj[rr][tx];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fmaf(zi[rr][ty * 4 + q], b, acc[q]);
+      const float4 a = *reinterpret_cast<const float4*>(&zi[rr][ty * 4]);
+      acc[0] = fmaf(a.x, b, acc[0]);
+      acc[1] = fmaf(a.y, b, acc[1]);
+      acc[2] = fmaf(a.z, b, acc[2]);
+      acc[3] = fmaf(a.w, b, acc[3]);
     }
     __syncthreads();
   }
@@ -96,7 +129,10 @@ __global__ void __launch_bounds__(256) cov_kernel(const float* __restrict__ x, i
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int i = i0 + ty * 4 + q, j = j0 + tx;
-    if (i < p && j < p) A[(long long)i * p + j] = acc[q] * inv;
+    if (i < p && j < p) {
+      A[(long long)i * p + j] = acc[q] * inv;
+      if (i0 != j0) A[(long long)j * p + i] = acc[q] * inv;
+    }
   }
 }
 
@@ -818,8 +854,9 @@ inline Workspace carve(void* ws, int p) {
 // the fit on a carved workspace (shared by the entry points)
 dk_status fit(dk_ctx* ctx, const float* x, int m, int p, int k, int sweeps, const Workspace& w, float* mean,
               float* scale, float* comps, float* eig, float* off_norm, cudaStream_t st) {
-  col_stats_kernel<<<(p + 31) / 32, 256, 0, st>>>(x, m, p, mean, scale);
-  cov_kernel<<<dim3((p + T32 - 1) / T32, (p + T32 - 1) / T32), 256, 0, st>>>(x, m, p, mean, scale, w.A);
+  col_stats_kernel<<<(p + 7) / 8, 64, 0, st>>>(x, m, p, mean, scale);
+  const int nt = (p + T32 - 1) / T32;
+  cov_kernel<<<nt * (nt + 1) / 2, 256, 0, st>>>(x, m, p, mean, scale, w.A);
   const int pe = p + (p & 1), np = pe / 2, rounds = sweeps * (pe - 1);
   const size_t mat_bytes = round256(size_t(p) * p * sizeof(float));
   const PersistPlan plan = persist_plan(p, ctx->sm_count, 2 * mat_bytes, mat_bytes);

@@ -509,9 +509,10 @@ using F32_P22r2 = GramCfg<float, 4, 1, 32, 2, 2, 1, 1, 2, 8>;     // 2 x 64 pair
 using F32_P11r1 = GramCfg<float, 4, 1, 32, 1, 1, 1, 1, 3, 16>;    // 1 x 32 pairs, one warp, 16 CTAs per SM
 using F32_P11w = GramCfg<float, 4, 4, 8, 1, 1, 1, 1, 4, 16>;      // 4 x 8 pairs, one warp, 16 CTAs per SM
 // FP64 issues at 2 multiply-adds a cycle and SM, so a tile's time is its pairs and the SMs in
-// use set the rate: one-warp tiles of 32 pairs. 64 samples at n = 8: 77 us, 36 us by the lanes
-// form (16 x 16 tiles with 256 threads: 142 us on 10 SMs).
-using F64_P11 = GramCfg<double, 4, 4, 8, 1, 1, 1, 1, 4, 8>;    // 4 x 8 pairs, one warp, 8 CTAs per SM
+// use set the rate (f64_small_tiles chooses). 64 samples at n = 8: 142 us with 16 x 16 tiles (10
+// SMs), 77 us with 4 x 8, 36 us by the lanes form.
+using F64_P11 = GramCfg<double, 4, 4, 8, 1, 1, 4, 2, 4, 1>;    // 16 x 16 pairs, 256 threads
+using F64_P11w = GramCfg<double, 4, 4, 8, 1, 1, 1, 1, 4, 8>;   // 4 x 8 pairs, one warp, 8 CTAs per SM
 using F32X8_P11 = GramCfg<float, 8, 4, 8, 1, 1, 4, 2, 4, 1>;   // chi = 8: 16 x 16 pairs, 256 threads
 using F32X8_S4 = GramCfg<float, 8, 4, 8, 1, 1, 4, 2, 2, 1, 4>;    // chi = 8: 16 x 16, 2 stages of 4 sites
 using F32X8_S2 = GramCfg<float, 8, 4, 8, 1, 1, 4, 2, 3, 1, 2>;    // chi = 8: 16 x 16, 3 stages of 2 sites
@@ -592,6 +593,22 @@ static const CfgInfo kF32Chi8[] = {info_of<F32X8_P11>(), info_of<F32X8_S4>(), in
 // bond-4 and bond-8 FP32 forms only where no tile shape is set).
 constexpr long long kLanesF32Chi4 = 40, kLanesF64Chi4 = 150, kLanesF32Chi8 = 50;
 
+// FP64: a warp instruction holds an SM's pipe 16 cycles, so a launch lasts as long as the SM with
+// the most warps' worth of tiles. 16 x 16 pairs are 8 of them, two such CTAs to an SM (whose tiles
+// come in pairs, therefore); they keep the pipe 94-100 % busy. 4 x 8 pairs are 1 and keep it 84-99 %
+// busy (three times the operand bytes per pair): taken where they are under 0.9 of the other's
+// count, i.e. where the last wave of the coarse tiles is mostly empty. n = 48, 4 x 8 against
+// 16 x 16, us: symmetric, 216 samples 621 (827), 260 samples 832 (1643), 352 samples 1463 (1647),
+// 379 samples 1886 (1647), 600 samples 4102 (4930), 2000 samples 42881 (42732); 1000 x 100
+// 2478 (3284), 1000 x 300 6598 (6579).
+static bool f64_small_tiles(const dk_ctx* ctx, const GramArgs& a) {
+  GramArgs t = a;
+  const long long sms = ctx->sm_count;
+  const long long coarse = 16 * ((count_tiles(t, F64_P11::TR, F64_P11::TC) + 2 * sms - 1) / (2 * sms));
+  const long long fine = (count_tiles(t, F64_P11w::TR, F64_P11w::TC) + sms - 1) / sms;
+  return 10 * fine < 9 * coarse;
+}
+
 // Pairs a block computes.
 static long long pair_count(const GramArgs& a) {
   const long long n = (long long)a.nrows * a.ncols;
@@ -633,7 +650,8 @@ static dk_status gram_dispatch(dk_ctx* ctx, const void* mps_r, int m_r, const vo
   if (dtype == DK_C128 && prec == DK_PREC_F64 && chi == 4 && pair_count(a) <= kLanesF64Chi4 * ctx->sm_count)
     return launch_lanes<double, 2, 2>(mps_r, m_r, mps_c, m_c, a, st);
   if (dtype == DK_C128 && prec == DK_PREC_F64 && chi == 4)
-    return launch_gram<F64_P11>(ctx, mps_r, m_r, mps_c, m_c, a, st);
+    return f64_small_tiles(ctx, a) ? launch_gram<F64_P11w>(ctx, mps_r, m_r, mps_c, m_c, a, st)
+                                   : launch_gram<F64_P11>(ctx, mps_r, m_r, mps_c, m_c, a, st);
   if (dtype == DK_C64 && prec == DK_PREC_F32 && chi == 8) {
     if (ctx->gram_config == 0 && pair_count(a) <= kLanesF32Chi8 * ctx->sm_count)
       return launch_lanes<float, 4, 2>(mps_r, m_r, mps_c, m_c, a, st);

@@ -283,7 +283,9 @@ __global__ void __launch_bounds__(256) jacobi_rotate_kernel(float* __restrict__ 
 //    between two buffers; a word of round q + 2 is written only after its CTA has read every
 //    angle of round q + 1, i.e. after every CTA has read those of round q. All waits are
 //    bounded; the launch is cooperative, so the CTAs run at the same time.
-// Up to about 130 features everything fits one CTA, and the angles pass through shared memory.
+// Below 64 features one CTA does it all, and the angles pass through shared memory: 0.57 against
+// 0.60 ms at p = 48 (10 sweeps), 0.76 against 0.73 at p = 64, 9.2 against 1.8 at p = 130, where one
+// CTA's rows and V^T take longer than a trip through L2.
 // The arithmetic and its order are those of jacobi_rotate_kernel: bit-identical results.
 // Bound by the latency of a round: the L2 round trip (about 950 cycles from a store to another
 // SM's load of it), the angle's divisions and roots (about 700 on one warp) and one barrier.
@@ -323,7 +325,7 @@ inline PersistPlan persist_plan(int p, int sms, size_t box_cap, size_t angle_cap
   };
   if (np <= 960 && size_t(32) * pe <= angle_cap) {
     const PersistPlan one = make(np);
-    if (one.smem <= SMEM_CAP) return one;
+    if (np < 32 && one.smem <= SMEM_CAP) return one;
     for (int ppc = 2; ppc < np; ++ppc) {
       const PersistPlan q = make(ppc);
       if (q.ctas > 1 && q.ctas <= sms && q.smem <= SMEM_CAP && q.box_bytes <= box_cap) return q;

@@ -159,24 +159,12 @@ __device__ inline void tables_f32(Coeffs& C, const float* xb, int bl, double ang
   double* hq = C.hq;
   double* jq = &C.jq[0][0];
   double* tv = &C.tv[0][0];
-  // The block's bl (bl + 1) / 2 angles, q <= r (q = r: the qubit's own), one per thread: an angle
-  // costs about 11 FP64 instructions, each of which holds the SM's FP64 pipe 16 cycles for a
-  // whole warp, so the angles are packed into as few warps as they fill. (Spread over the 12 x 12
-  // table they took 4.5 warps' time for 2.) The tables below
-  // read q < r only.
-  for (int e = tid; e < bl * (bl + 1) / 2; e += nt) {
-    int q = 0, r = e;
-    while (r >= bl - q) {
-      r -= bl - q;
-      ++q;
-    }
-    r += q;
-    const bool on = q == r || pairs_kind == DK_ENT_FULL || (pairs_kind == DK_ENT_CHAIN && r == q + 1);
-    uint32_t turns = 0u;
-    if (on)
-      turns = turns32(q == r ? 0.5 * angle_scale * double(xb[q]) : (PI_D - double(xb[q])) * (PI_D - double(xb[r])));
-    if (q == r) slot(hq, q) = turns;
-    else slot(jq, q * MAXB + r) = turns;
+  if (tid < bl) slot(hq, tid) = turns32(0.5 * angle_scale * double(xb[tid]));
+  for (int e = tid; e < MAXB * MAXB; e += nt) {
+    const int q = e / MAXB, r = e % MAXB;
+    const bool on = q < bl && r < bl && q < r &&
+                    (pairs_kind == DK_ENT_FULL || (pairs_kind == DK_ENT_CHAIN && r == q + 1));
+    slot(jq, e) = on ? turns32((PI_D - double(xb[q])) * (PI_D - double(xb[r]))) : 0u;
   }
   sync();
   // tables: z of qubit q (q < hb) is bit hb-1-q of zH; of qubit hb+t is bit lb-1-t of zL

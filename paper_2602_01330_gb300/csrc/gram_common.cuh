@@ -34,26 +34,9 @@ struct GramArgs {
 // tile (ti, tj) covers rows from ti*TR and columns up to (tj+1)*TC - 1.
 __host__ __device__ __forceinline__ int first_upper_tile(int ti, int tr, int tc) { return (ti * tr) / tc; }
 
-// Tile index t (row-major over the tiles that are computed) -> (row tile, column tile). Symmetric:
-// K = tc / tr row tiles (one if tr >= tc) share a first column tile, which moves on by R = tr / tc
-// (one if tc >= tr) from one group of them to the next, so K (g tiles_c - R g (g - 1) / 2) tiles
-// come before group g: g is the root of a quadratic, put right by whole-number steps. (A walk
-// over the rows, once per tile and again for each stage loaded ahead of it, was 6 % of the
-// 2000 x 2000 Gram at n = 16.)
-__host__ __device__ __forceinline__ void decode_tile(const GramArgs& p, int tr, int tc, int t, int& ti, int& tj) {
-  if (p.symmetric && (tr % tc == 0 || tc % tr == 0)) {
-    const int K = tc > tr ? tc / tr : 1, R = tr > tc ? tr / tc : 1;
-    auto before = [&](int g) { return (long long)K * ((long long)g * p.tiles_c - (long long)R * ((long long)g * (g - 1) / 2)); };
-    const float b = float(p.tiles_c) + 0.5f * float(R);
-    int g = int((b - sqrtf(fmaxf(b * b - float(2 * R) * (float(t) / float(K)), 0.0f))) / float(R));
-    const int last = (p.tiles_c - 1) / R;  // the last group with a tile
-    g = g < 0 ? 0 : g > last ? last : g;
-    while (g < last && before(g + 1) <= t) ++g;
-    while (g > 0 && before(g) > t) --g;
-    const int cnt = p.tiles_c - g * R, o = int(t - before(g)), row = o / cnt;
-    ti = g * K + row;
-    tj = g * R + o - row * cnt;
-  } else if (p.symmetric) {
+// Tile index t (row-major over the tiles that are computed) -> (row tile, column tile).
+__device__ __forceinline__ void decode_tile(const GramArgs& p, int tr, int tc, int t, int& ti, int& tj) {
+  if (p.symmetric) {
     int r = 0;
     while (true) {
       const int first = first_upper_tile(r, tr, tc);
@@ -69,6 +52,30 @@ __host__ __device__ __forceinline__ void decode_tile(const GramArgs& p, int tr, 
   } else {
     ti = t / p.tiles_c;
     tj = t - ti * p.tiles_c;
+  }
+}
+
+// The same without a walk over the rows, for kernels of many small tiles. Symmetric:
+// K = tc / tr row tiles (one if tr >= tc) share a first column tile, which moves on by R = tr / tc
+// (one if tc >= tr) from one group of them to the next, so K (g tiles_c - R g (g - 1) / 2) tiles
+// come before group g: g is the root of a quadratic, put right by whole-number steps. (A walk
+// over the rows, once per tile and again for each stage loaded ahead of it, was 6 % of the
+// 2000 x 2000 Gram at n = 16.)
+__device__ __forceinline__ void decode_small_tile(const GramArgs& p, int tr, int tc, int t, int& ti, int& tj) {
+  if (p.symmetric && (tr % tc == 0 || tc % tr == 0)) {
+    const int K = tc > tr ? tc / tr : 1, R = tr > tc ? tr / tc : 1;
+    auto before = [&](int g) { return (long long)K * ((long long)g * p.tiles_c - (long long)R * ((long long)g * (g - 1) / 2)); };
+    const float b = float(p.tiles_c) + 0.5f * float(R);
+    int g = int((b - sqrtf(fmaxf(b * b - float(2 * R) * (float(t) / float(K)), 0.0f))) / float(R));
+    const int last = (p.tiles_c - 1) / R;  // the last group with a tile
+    g = g < 0 ? 0 : g > last ? last : g;
+    while (g < last && before(g + 1) <= t) ++g;
+    while (g > 0 && before(g) > t) --g;
+    const int cnt = p.tiles_c - g * R, o = int(t - before(g)), row = o / cnt;
+    ti = g * K + row;
+    tj = g * R + o - row * cnt;
+  } else {
+    decode_tile(p, tr, tc, t, ti, tj);
   }
 }
 

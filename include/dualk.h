@@ -457,7 +457,7 @@ dk_status dk_dual_kernel_rows(dk_ctx* ctx,
  *                 one chain instead of three — the choice when many entries exceed tau; NULL
  *                 (ws_bytes ignored): each entry computes both of its norms. Both give the
  *                 same values. Nothing is read from ws before it is written.
- * Bond 4 / 8: one thread per refined entry (queued per warp); bond 32: one warp per entry
+ * Bond 4 / 8: 8 lanes / one warp per refined entry (queued per warp); bond 32: one warp per entry
  * (chains of about 1e9 operations each), so the cost is proportional to the number of
  * entries above tau: nothing but reads of the block when there are none.
  * Errors: DK_ERR_ARG (NULL pointers, ranges, ld < ncols, neither kq_out nor logkq_out, tau

@@ -58,9 +58,9 @@ __device__ __forceinline__ void decode_tile(const GramArgs& p, int tr, int tc, i
 // The same without a walk over the rows, for kernels of many small tiles. Symmetric:
 // K = tc / tr row tiles (one if tr >= tc) share a first column tile, which moves on by R = tr / tc
 // (one if tc >= tr) from one group of them to the next, so K (g tiles_c - R g (g - 1) / 2) tiles
-// come before group g: g is the root of a quadratic, put right by whole-number steps. (A walk
-// over the rows, once per tile and again for each stage loaded ahead of it, was 6 % of the
-// 2000 x 2000 Gram at n = 16.)
+// come before group g: g is the root of a quadratic, put right by whole-number steps. 2000 x 2000
+// at n = 16: 332 us, with a walk over the rows, once per tile and again for each stage loaded
+// ahead of it, 369 us; kernels of 128 x 128 tiles, whose walk is short, lose 25 us a launch by it.
 __device__ __forceinline__ void decode_small_tile(const GramArgs& p, int tr, int tc, int t, int& ti, int& tj) {
   if (p.symmetric && (tr % tc == 0 || tc % tr == 0)) {
     const int K = tc > tr ? tc / tr : 1, R = tr > tc ? tr / tc : 1;

@@ -27,6 +27,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "jacobi_ring.h"
 
 namespace dk {
 namespace pca {
@@ -280,9 +281,14 @@ __global__ void __launch_bounds__(256) jacobi_rotate_kernel(float* __restrict__ 
 //    row where it stands next, so one barrier a round is enough.
 //  * Everything in transit is a 16-byte word with a round tag, stored and loaded as one: the tag
 //    says that the values are there, so there is no barrier and no fence. Words alternate
-//    between two buffers; a word of round q + 2 is written only after its CTA has read every
-//    angle of round q + 1, i.e. after every CTA has read those of round q. All waits are
-//    bounded; the launch is cooperative, so the CTAs run at the same time.
+//    between two buffers. Every CTA publishes at least one word in every round and every CTA
+//    waits for all of them (ring_publishes says why; the pair of an odd p's padding index has
+//    its word too, and a last CTA of one pair always sends one, for which a thread of its own
+//    waits). A CTA publishes for round q + 1 only when it has read all words of round q, so a
+//    CTA that has all words of round q + 1 and writes over those of round q knows that every
+//    other one has read them. The rows' words need only that neighbours send to each other in
+//    every round. All waits are bounded; the launch is cooperative, so the CTAs run at the same
+//    time.
 // Below 64 features one CTA does it all, and the angles pass through shared memory: 0.57 against
 // 0.60 ms at p = 48 (10 sweeps), 0.76 against 0.73 at p = 64, 9.2 against 1.8 at p = 130, where one
 // CTA's rows and V^T take longer than a trip through L2.
@@ -291,48 +297,6 @@ __global__ void __launch_bounds__(256) jacobi_rotate_kernel(float* __restrict__ 
 // SM's load of it), the angle's divisions and roots (about 700 on one warp) and one barrier.
 // Measured, 10 sweeps at p = 784 (131 CTAs of 3 row pairs): 13.2 ms, 1.7 us a round, against
 // 79.4 ms with one launch per round (10.1 us).
-
-constexpr int UR = 4;  // row pairs of a thread in flight
-
-struct PersistPlan {
-  int ctas, ppc, vc, threads;  // vc: columns of V^T per CTA
-  size_t smem, box_bytes;
-};
-
-// Box memory (16-byte words): for several CTAs the rows in transit (2 buffers x CTAs x 2 rows x
-// np column pairs), then the published angles (2 buffers x pe). It ends with V^T's part of the
-// workspace, which is written only at the end, and reaches back into A's: the first row is
-// sent in round 0 by a CTA that has everybody's angles, i.e. after every CTA has read its part
-// of A. The fewest pairs per CTA that this and the SM count allow: a CTA's work on its rows is
-// what a round waits for.
-inline PersistPlan persist_plan(int p, int sms, size_t box_cap, size_t angle_cap) {
-  const int pe = p + (p & 1), np = pe / 2;
-  const int lanes = (np + 31) / 32 * 32;  // one thread per column pair, groups of them over the rows
-  constexpr size_t SMEM_CAP = 220 * 1024;
-  auto make = [&](int ppc) {
-    PersistPlan q;
-    q.ppc = ppc;
-    q.ctas = (np + ppc - 1) / ppc;
-    q.vc = (p + q.ctas - 1) / q.ctas;
-    // a thread per column pair, in groups over the row pairs when there are more than UR of
-    // these, and warps of their own for the elements that the next round waits for
-    const int side = (2 * ppc + 31) / 32 * 32, room = (1024 - side) / lanes, want = (ppc + UR - 1) / UR;
-    q.threads = lanes * (room < want ? room : want) + side;
-    q.smem = size_t((q.vc + 3) / 4) * pe * 16 + size_t(2) * np * 16 + size_t(pe) * 16 + size_t(4) * ppc * pe * 4 +
-             size_t(pe) * 4;
-    q.box_bytes = size_t(32) * pe + (q.ctas > 1 ? size_t(32) * q.ctas * pe : 0);
-    return q;
-  };
-  if (np <= 960 && size_t(32) * pe <= angle_cap) {
-    const PersistPlan one = make(np);
-    if (np < 32 && one.smem <= SMEM_CAP) return one;
-    for (int ppc = 2; ppc < np; ++ppc) {
-      const PersistPlan q = make(ppc);
-      if (q.ctas > 1 && q.ctas <= sms && q.smem <= SMEM_CAP && q.box_bytes <= box_cap) return q;
-    }
-  }
-  return PersistPlan{0, 0, 0, 0, 0, 0};
-}
 
 struct PersistArgs {
   float* A;
@@ -387,7 +351,7 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
   const int G = int(gridDim.x), g = int(blockIdx.x), NT = int(blockDim.x), tid = int(threadIdx.x);
   const int ks = g * a.ppc, ke = min(ks + a.ppc, np), cnt = ke - ks;
   const int v0 = g * a.vc, vn = max(0, min(a.vc, p - v0)), vp = (a.vc + 3) / 4;
-  const bool solo = G == 1;
+  const bool solo = G == 1, lone = ring_lone(np, a.ppc);
   // shared memory: V^T columns [plane][row][4], angles [2 rounds][pair] (c, s, t), solo: the
   // published angles by x, rows [2 rounds][local row][pe], the diagonal of A
   float4* V = reinterpret_cast<float4*>(sm);
@@ -399,15 +363,11 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
   uint4* wR = a.words;                                              // [buffer][CTA][upper / lower][np]
   uint4* wN = wR + (solo ? 0 : size_t(4) * G * np);                 // [buffer][pe]
   auto box = [&](int buf, int cta, int which) { return wR + (size_t(buf * G + cta) * 2 + which) * np; };
-  auto idx_at = [&](int t, int r) {  // index at position t in round r
-    int x = t - 1 + r;
-    if (x >= ring) x -= ring;
-    return t == 0 ? 0 : 1 + x;
-  };
-  auto came_from = [&](int t) { return t == 0 ? 0 : (t == ring ? 1 : t + 1); };  // its position a round earlier
-  auto goes_to = [&](int t) { return t == 0 ? 0 : (t == 1 ? ring : t - 1); };
+  auto idx_at = [&](int t, int r) { return ring_index(t, r, ring); };
+  auto came_from = [&](int t) { return ring_came_from(t, ring); };
+  auto goes_to = [&](int t) { return ring_goes_to(t, ring); };
   // local row u < cnt: position ks + u; u >= cnt: position pe - ke + (u - cnt)
-  auto pos_of = [&](int u) { return u < cnt ? ks + u : pe - ke + (u - cnt); };
+  auto pos_of = [&](int u) { return ring_row_position(u, ks, ke, pe); };
   auto row_at = [&](int t) { return t < np ? t - ks : cnt + t - (pe - ke); };
   // where local row u stands next; -1: at another CTA
   auto moves_to = [&](int u) {
@@ -430,16 +390,16 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
   __syncthreads();  // what this CTA reads of A is read: only now does it publish anything
   for (int u = tid; u < 2 * cnt; u += NT) {
     const int i = pos_of(u), j = ring - i;  // round 0: index = position
-    if (i < j && j < p) {
-      const float o = rows[u * pe + j];
-      const float4 w = pair_rotation(sD[i], sD[j], o);
+    if (i < j) {
+      const float o = j < p ? rows[u * pe + j] : 0.0f;
+      const float4 w = j < p ? pair_rotation(sD[i], sD[j], o) : make_float4(1.0f, 0.0f, 0.0f, 0.0f);
       if (solo) sN[i] = make_float4(w.x, w.z, o, 0.0f);
       else put_word(wN + i, w.x, w.z, o, tag_of(0));
     }
   }
   __syncthreads();
 
-  const int side = (2 * a.ppc + 31) / 32 * 32, workers = NT - side;
+  const int side = ring_side_threads(a.ppc, np), workers = NT - side;
   const int copy = 2 * a.ppc * pe;  // floats between the two copies of the rows
   const bool can_up = g < G - 1, can_low = g > 0;
   if (tid >= workers) {
@@ -447,23 +407,32 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
     const int u = tid - workers;
     const bool holds = u < 2 * cnt;
     const int hu = holds ? (u < cnt ? u : 2 * cnt - 1 - u) : 0;
-    const int ty = holds ? came_from(ring - goes_to(pos_of(u))) : 0, kc = min(ty, ring - ty);
+    const int tx = holds ? pos_of(u) : 0, ty = holds ? came_from(ring - goes_to(tx)) : 0, kc = min(ty, ring - ty);
+    const bool watches = lone && u == 2 * a.ppc;  // waits for the lone CTA's word
     int r = 0;
     for (int q = 0; q < a.rounds; ++q) {
       const int buf = q & 1;
-      const int x = holds ? idx_at(pos_of(u), r) : 0, y = idx_at(ty, r), z = idx_at(ring - ty, r);
+      const int x = idx_at(tx, r), y = idx_at(ty, r), z = idx_at(ring - ty, r);
       const bool up = idx_at(ks + hu, r) < idx_at(ring - ks - hu, r), low = y < z;
       const float* ri = rows + buf * copy + (up ? hu : 2 * cnt - 1 - hu) * pe;
       const float* rj = rows + buf * copy + (up ? 2 * cnt - 1 - hu : hu) * pe;
       const int c0 = low ? y : z, c1 = low ? z : y;
       const bool is_i = (u < cnt) == up;
+      if (watches) {
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (!await_word(w, wN + buf * pe + ring_lone_index(np, r, ring), tag_of(q))) s_abort = 1;
+      }
       __syncthreads();
       if (s_abort) break;
-      if (q + 1 < a.rounds && holds && y > x && y < p) {  // otherwise the partner's owner does it
-        float b00 = ri[c0], b01 = ri[c1], b10 = rj[c0], b11 = rj[c1];
-        rotate_block(pars[buf * np + ks + hu], pars[buf * np + kc], ks + hu == kc, b00, b01, b10, b11);
-        const float o = is_i ? (low ? b00 : b01) : (low ? b10 : b11);
-        const float4 w = pair_rotation(sD[x], sD[y], o);
+      if (q + 1 < a.rounds && holds && ring_publishes(x, y, tx, np, lone)) {  // otherwise the partner's owner does
+        float o = 0.0f;
+        float4 w = make_float4(1.0f, 0.0f, 0.0f, 0.0f);
+        if (y > x && (!ODD || y < p)) {
+          float b00 = ri[c0], b01 = ri[c1], b10 = rj[c0], b11 = rj[c1];
+          rotate_block(pars[buf * np + ks + hu], pars[buf * np + kc], ks + hu == kc, b00, b01, b10, b11);
+          o = is_i ? (low ? b00 : b01) : (low ? b10 : b11);
+          w = pair_rotation(sD[x], sD[y], o);
+        }
         if (solo) sN[x] = make_float4(w.x, w.z, o, 0.0f);
         else put_word(wN + (buf ^ 1) * pe + x, w.x, w.z, o, tag_of(q + 1));
       }
@@ -522,6 +491,7 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
       // (the ends of the upper run, from CTA g + 1, and of the lower one, from g - 1)
       float4 r2 = make_float4(1.0f, 0.0f, 0.0f, 0.0f);
       if (grp == 0 && active) {
+        if (!solo) ok = await_word(wn, wN + buf * pe + i2, tag) && ok;  // the padding index's pair too
         if (has_j2) {
           float o;
           if (solo) {
@@ -530,7 +500,6 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
             r2.z = v.y;
             o = v.z;
           } else {
-            ok = await_word(wn, wN + buf * pe + i2, tag) && ok;
             r2.x = __uint_as_float(wn.x);
             r2.z = __uint_as_float(wn.y);
             o = __uint_as_float(wn.z);

@@ -834,8 +834,11 @@ dk_status fit(dk_ctx* ctx, const float* x, int m, int p, int k, int sweeps, cons
   if (cudaMemsetAsync(w.done, 0, sizeof(unsigned), st) != cudaSuccess) return DK_ERR_CUDA;
   bool persistent = false;
   if (plan.ctas > 0) {
-    // no word of V^T's part, which a former call may have used, has a tag yet
-    if (cudaMemsetAsync(w.Vt, 0, mat_bytes, st) != cudaSuccess) return DK_ERR_CUDA;
+    // no word after the covariance (A's padding and V^T's part), which a former call may have used,
+    // has a tag yet
+    const size_t cov_bytes = size_t(p) * p * sizeof(float);
+    if (cudaMemsetAsync(reinterpret_cast<uint8_t*>(w.A) + cov_bytes, 0, 2 * mat_bytes - cov_bytes, st) != cudaSuccess)
+      return DK_ERR_CUDA;
     uint8_t* box = reinterpret_cast<uint8_t*>(w.Vt) + mat_bytes - plan.box_bytes;
     const bool odd = p & 1, small = plan.threads <= 512;
     const void* kern = odd ? (small ? reinterpret_cast<const void*>(jacobi_persist_kernel<512, true>)
@@ -963,9 +966,9 @@ DK_API dk_status dk_pca_fit_noalloc(dk_ctx* ctx, const float* x, int m, int p, i
   void* scratch = nullptr;
   const dk_status s = pca::noalloc_scratch(ctx->device, &scratch);
   if (s != DK_OK) return s;
-  // every part of the scratch that the fit reads is written earlier in the same call (the
-  // covariance, the identity, each round's rotation table, the round counter, which the fit
-  // clears), so nothing else needs clearing
+  // every part of the scratch that the fit reads is written earlier in the same call: the
+  // covariance, the identity or the words of the one-launch form (whose place the fit clears), each
+  // round's rotation table, the round counter, which the fit clears
   return pca::fit(ctx, x, m, p, k, sweeps, pca::carve(scratch, p), mean, scale, components, eigenvalues, off_norm,
                   static_cast<cudaStream_t>(stream));
 }

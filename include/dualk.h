@@ -523,6 +523,8 @@ size_t dk_pca_workspace_bytes(int p);
  *   off_norm     1 float (device, written, may be NULL): sqrt(off-diagonal / total sum of
  *                squares) of the rotated covariance after the last sweep (about 1e-7 when
  *                the sweeps sufficed)
+ * If a device-side wait of the rounds runs out, dk_sync_status gives DK_ERR_TIMEOUT, and
+ * components, eigenvalues and off_norm are NaN.
  * Errors: DK_ERR_ARG (NULL pointers, m < 2, p < 2, k outside 1..p, sweeps outside 1..100),
  *         DK_ERR_UNSUPPORTED (p > DK_PCA_MAX_FEATURES), DK_ERR_WORKSPACE (workspace too small
  *         or misaligned). */

@@ -303,6 +303,7 @@ struct PersistArgs {
   float* Vt;
   uint4* words;  // box memory
   unsigned* done;
+  unsigned* failed;
   unsigned* status;
   int p, ppc, vc, rounds;
 };
@@ -625,7 +626,10 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
     __syncthreads();
   }
   if (s_abort) {
-    if (tid == 0) record_status(a.status, DEV_TIMEOUT);
+    if (tid == 0) {
+      record_status(a.status, DEV_TIMEOUT);
+      *a.failed = 1u;  // A and V^T are not a result: the outputs become NaN
+    }
     return;
   }
   const int rl = (a.rounds - 1) % ring;  // rows stand where the last round had them
@@ -665,6 +669,7 @@ __global__ void __launch_bounds__(256) off_norm_kernel(const float* __restrict__
 }
 
 __global__ void __launch_bounds__(32) off_norm_finish_kernel(const double2* __restrict__ part, int n,
+                                                             const unsigned* __restrict__ failed,
                                                              float* __restrict__ out) {
   double off = 0.0, all = 0.0;
   for (int e = threadIdx.x; e < n; e += 32) {
@@ -676,14 +681,22 @@ __global__ void __launch_bounds__(32) off_norm_finish_kernel(const double2* __re
     off += __shfl_xor_sync(0xffffffffu, off, o);
     all += __shfl_xor_sync(0xffffffffu, all, o);
   }
-  if (threadIdx.x == 0) *out = all > 0.0 ? float(sqrt(off / all)) : 0.0f;
+  if (threadIdx.x == 0) *out = *failed ? NAN : all > 0.0 ? float(sqrt(off / all)) : 0.0f;
 }
 
 // block i: the rank of eigenvalue A_ii among all (decreasing, smaller index first on ties);
-// if below k, row rank of the output is row i of V^T with the sign of its largest entry
+// if below k, row rank of the output is row i of V^T with the sign of its largest entry. All NaN if
+// the rounds gave up.
 __global__ void __launch_bounds__(256) select_kernel(const float* __restrict__ A, const float* __restrict__ Vt, int p,
-                                                     int k, float* __restrict__ comps, float* __restrict__ eig) {
+                                                     int k, const unsigned* __restrict__ failed,
+                                                     float* __restrict__ comps, float* __restrict__ eig) {
   const int i = blockIdx.x;
+  if (*failed) {
+    if (i >= k) return;
+    for (int c = threadIdx.x; c < p; c += 256) comps[(long long)i * p + c] = NAN;
+    if (threadIdx.x == 0) eig[i] = NAN;
+    return;
+  }
   const float li = A[(long long)i * p + i];
   __shared__ int s_rank[256];
   __shared__ float s_best[256];
@@ -795,7 +808,8 @@ struct Workspace {
   float* Vt;
   int2* ij;
   float4* cs;
-  unsigned* done;  // CTAs finished in the current Jacobi round
+  unsigned* done;    // CTAs finished in the current Jacobi round
+  unsigned* failed;  // a wait of the one-launch form ran out
 };
 
 inline size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -819,19 +833,26 @@ inline Workspace carve(void* ws, int p) {
   w.cs = reinterpret_cast<float4*>(b);
   b += round256(pe / 2 * sizeof(float4));
   w.done = reinterpret_cast<unsigned*>(b);
+  w.failed = w.done + 1;
   return w;
 }
 
-// the fit on a carved workspace (shared by the entry points)
-dk_status fit(dk_ctx* ctx, const float* x, int m, int p, int k, int sweeps, const Workspace& w, float* mean,
-              float* scale, float* comps, float* eig, float* off_norm, cudaStream_t st) {
+inline PersistPlan plan_of(const dk_ctx* ctx, int p) {
+  const size_t mat_bytes = round256(size_t(p) * p * sizeof(float));
+  return persist_plan(p, ctx->sm_count, 2 * mat_bytes, mat_bytes);
+}
+
+// the fit on a carved workspace (shared by the entry points); plan: plan_of's, or one of no CTAs for a
+// launch per round
+dk_status fit(dk_ctx* ctx, const float* x, int m, int p, int k, int sweeps, const Workspace& w,
+              const PersistPlan& plan, float* mean, float* scale, float* comps, float* eig, float* off_norm,
+              cudaStream_t st) {
   col_stats_kernel<<<(p + 7) / 8, 64, 0, st>>>(x, m, p, mean, scale);
   const int nt = (p + T32 - 1) / T32;
   cov_kernel<<<nt * (nt + 1) / 2, 256, 0, st>>>(x, m, p, mean, scale, w.A);
   const int pe = p + (p & 1), np = pe / 2, rounds = sweeps * (pe - 1);
   const size_t mat_bytes = round256(size_t(p) * p * sizeof(float));
-  const PersistPlan plan = persist_plan(p, ctx->sm_count, 2 * mat_bytes, mat_bytes);
-  if (cudaMemsetAsync(w.done, 0, sizeof(unsigned), st) != cudaSuccess) return DK_ERR_CUDA;
+  if (cudaMemsetAsync(w.done, 0, 2 * sizeof(unsigned), st) != cudaSuccess) return DK_ERR_CUDA;  // and failed
   bool persistent = false;
   if (plan.ctas > 0) {
     // no word after the covariance (A's padding and V^T's part), which a former call may have used,
@@ -847,8 +868,8 @@ dk_status fit(dk_ctx* ctx, const float* x, int m, int p, int k, int sweeps, cons
                                     : reinterpret_cast<const void*>(jacobi_persist_kernel<1024, false>));
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(plan.smem)) != cudaSuccess)
       return DK_ERR_CUDA;
-    PersistArgs a{w.A,  w.Vt, reinterpret_cast<uint4*>(box), w.done, ctx->status, p, plan.ppc, plan.vc,
-                  rounds};
+    PersistArgs a{w.A,  w.Vt, reinterpret_cast<uint4*>(box), w.done, w.failed, ctx->status, p, plan.ppc,
+                  plan.vc, rounds};
     void* args[] = {&a};
     persistent = cudaLaunchCooperativeKernel(kern, dim3(plan.ctas), dim3(plan.threads), args, plan.smem, st) ==
                  cudaSuccess;
@@ -868,9 +889,9 @@ dk_status fit(dk_ctx* ctx, const float* x, int m, int p, int k, int sweeps, cons
     // the rotation table is done with: it holds the partial sums, one 16-byte entry per CTA
     double2* part = reinterpret_cast<double2*>(w.cs);
     off_norm_kernel<<<np, 256, 0, st>>>(w.A, p, part);
-    off_norm_finish_kernel<<<1, 32, 0, st>>>(part, np, off_norm);
+    off_norm_finish_kernel<<<1, 32, 0, st>>>(part, np, w.failed, off_norm);
   }
-  select_kernel<<<p, 256, 0, st>>>(w.A, w.Vt, p, k, comps, eig);
+  select_kernel<<<p, 256, 0, st>>>(w.A, w.Vt, p, k, w.failed, comps, eig);
   return launch_status();
 }
 
@@ -889,8 +910,8 @@ DK_API dk_status dk_pca_fit(dk_ctx* ctx, const float* x, int m, int p, int k, in
   if (p > DK_PCA_MAX_FEATURES) return DK_ERR_UNSUPPORTED;
   if (workspace_bytes < pca::workspace_bytes(p) || (reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
     return DK_ERR_WORKSPACE;
-  return pca::fit(ctx, x, m, p, k, sweeps, pca::carve(workspace, p), mean, scale, components, eigenvalues,
-                  off_norm, static_cast<cudaStream_t>(stream));
+  return pca::fit(ctx, x, m, p, k, sweeps, pca::carve(workspace, p), pca::plan_of(ctx, p), mean, scale, components,
+                  eigenvalues, off_norm, static_cast<cudaStream_t>(stream));
 }
 
 DK_API dk_status dk_pca_transform(dk_ctx* ctx, const float* x, int m, int p, const float* mean, const float* scale,
@@ -969,6 +990,6 @@ DK_API dk_status dk_pca_fit_noalloc(dk_ctx* ctx, const float* x, int m, int p, i
   // every part of the scratch that the fit reads is written earlier in the same call: the
   // covariance, the identity or the words of the one-launch form (whose place the fit clears), each
   // round's rotation table, the round counter, which the fit clears
-  return pca::fit(ctx, x, m, p, k, sweeps, pca::carve(scratch, p), mean, scale, components, eigenvalues, off_norm,
-                  static_cast<cudaStream_t>(stream));
+  return pca::fit(ctx, x, m, p, k, sweeps, pca::carve(scratch, p), pca::plan_of(ctx, p), mean, scale, components,
+                  eigenvalues, off_norm, static_cast<cudaStream_t>(stream));
 }

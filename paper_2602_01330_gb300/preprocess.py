@@ -22,9 +22,15 @@ class PCAPreprocessor:
         self.model = None
 
     def fit(self, x_train: torch.Tensor):
-        """Standardisation and PCA on the raw training rows (m x p float32, CUDA)."""
+        """Standardisation and PCA on the raw training rows (m x p float32, CUDA). Waits for the
+        fit and raises if one of its device-side waits ran out (its outputs are NaN then, which
+        the min-max scaling would turn into zeros); inside a stream capture, where nothing has
+        run yet, that check is the caller's."""
         k = self.k_max or x_train.shape[1]
-        self.model = dualk.pca_fit(self.ctx, x_train.contiguous(), k, self.sweeps)
+        model = dualk.pca_fit(self.ctx, x_train.contiguous(), k, self.sweeps)
+        if not torch.cuda.is_current_stream_capturing():
+            self.ctx.sync_status()
+        self.model = model
         return self
 
     def features(self, x_train: torch.Tensor, x_test: torch.Tensor, n: int):

@@ -590,8 +590,8 @@ constexpr int kF32Chi8Default = 2;  // 16 x 16 pairs, 2 stages of 4 sites: faste
 static const CfgInfo kF32Chi8[] = {info_of<F32X8_P11>(), info_of<F32X8_S4>(), info_of<F32X8_S2>(),
                                    info_of<F32X8_h>(), info_of<F32X8_q>()};
 
-// Pairs per SM up to which gram_lanes_kernel takes a block: between the sizes measured there (the
-// bond-4 and bond-8 FP32 forms only where no tile shape is set).
+// Pairs per SM up to which gram_lanes_kernel takes a block where no tile shape is set: between the
+// sizes measured there.
 constexpr long long kLanesF32Chi4 = 40, kLanesF64Chi4 = 150, kLanesF32Chi8 = 50;
 
 // FP64: a warp instruction holds an SM's pipe 16 cycles, so a launch lasts as long as the SM with
@@ -648,11 +648,14 @@ static dk_status gram_dispatch(dk_ctx* ctx, const void* mps_r, int m_r, const vo
       default: return launch_gram<F32_P22qS6>(ctx, mps_r, m_r, mps_c, m_c, a, st);
     }
   }
-  if (dtype == DK_C128 && prec == DK_PREC_F64 && chi == 4 && pair_count(a) <= kLanesF64Chi4 * ctx->sm_count)
-    return launch_lanes<double, 2, 2>(mps_r, m_r, mps_c, m_c, a, st);
-  if (dtype == DK_C128 && prec == DK_PREC_F64 && chi == 4)
+  if (dtype == DK_C128 && prec == DK_PREC_F64 && chi == 4) {
+    // a shape that is set: the one of the complex128 table, also for an id beyond it
+    if (ctx->gram_config > 0) return launch_gram<F64_P11>(ctx, mps_r, m_r, mps_c, m_c, a, st);
+    if (pair_count(a) <= kLanesF64Chi4 * ctx->sm_count)
+      return launch_lanes<double, 2, 2>(mps_r, m_r, mps_c, m_c, a, st);
     return f64_small_tiles(ctx, a) ? launch_gram<F64_P11w>(ctx, mps_r, m_r, mps_c, m_c, a, st)
                                    : launch_gram<F64_P11>(ctx, mps_r, m_r, mps_c, m_c, a, st);
+  }
   if (dtype == DK_C64 && prec == DK_PREC_F32 && chi == 8) {
     if (ctx->gram_config == 0 && pair_count(a) <= kLanesF32Chi8 * ctx->sm_count)
       return launch_lanes<float, 4, 2>(mps_r, m_r, mps_c, m_c, a, st);

@@ -1,0 +1,57 @@
+"""A tile shape that a caller sets is the one that runs, in every precision that has shapes: the
+threads per CTA of the captured launch are those that dk_gram_config_info reports."""
+import ctypes
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+class _KernelNode(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS_v2
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3),
+                ("smem", ctypes.c_uint), ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def _launched_threads(torch, call):
+    """Threads per CTA of each kernel that `call` launches, from a capture of it."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    call()  # lazy loading and workspaces before the capture
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        call()
+    graph = ctypes.c_void_p(g.raw_cuda_graph())
+    n = ctypes.c_size_t(0)
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    threads = []
+    for node in nodes:
+        kind, par = ctypes.c_int(-1), _KernelNode()
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value == 0:  # CU_GRAPH_NODE_TYPE_KERNEL
+            assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(par)) == 0
+            threads.append(par.block[0])
+    return threads
+
+
+# 40 samples: few enough for the lanes form; 230: where the built-in choice is the small FP64 tiles
+@pytest.mark.parametrize("m", [40, 230])
+@pytest.mark.parametrize("c128,chi,cid", [(True, 4, 1), (False, 4, 1), (False, 4, 17), (False, 4, 22), (False, 8, 1)])
+def test_set_shape_runs(c128, chi, cid, m):
+    import torch
+    from paper_2602_01330_gb300 import build, dualk, synthetic
+    build.build()
+    ctx = dualk.Context(0)
+    dtype = dualk.DK_C128 if c128 else dualk.DK_C64
+    x = torch.from_numpy(synthetic.uniform_angles(m, 6, seed=9, dtype=np.float32)).cuda()
+    mps = dualk.mps_build(ctx, x, dualk.FeatureMap(reps=3 if chi == 8 else 2, chi_max=chi), dtype=dtype)
+    ctx.set_gram_config(cid)
+    _, _, threads = dualk.gram_config_info(cid, dtype, chi)
+    got = _launched_threads(torch, lambda: dualk.gram(ctx, mps, refine=None))
+    ctx.set_gram_config(0)
+    assert got == [threads]
+    ctx.sync_status()
+    ctx.close()

@@ -545,23 +545,26 @@ static const CfgInfo kF32Chi4[] = {info_of<F32_P11>(),  info_of<F32_P21>(),  inf
 constexpr int kF32Chi4Default = 17;  // 16 x 16 pairs, 4 CTAs per SM, 6-site stages: fastest where tiles fill many waves
 
 // The built-in complex64 / chi 4 shape for a block: the least estimated time over a few shapes,
-// from what a site costs a wave of CTAs in ns, measured at n = 784 against 8000 columns: `full`
-// a full wave, `low` one with at most per_low CTAs per SM (a warp per scheduler; for shape 17
-// two CTAs often share two schedulers), equal steps of per_low CTAs in between. Few rows leave
-// most of a 16-row tile empty, and a wave of four-pair threads takes the chain's latency however
-// few CTAs it has, so small blocks take narrower tiles and one pair per thread. Measured, us,
-// against shape 17: 8000 columns at n = 784 with 1 row 446 (1126), 5 rows 725 (1127), 37 rows
-// 2546 (3272), 100 rows 6430 (6613); symmetric 40 samples 417 (614). Where shape 17 needs 8
-// waves or more its last one matters little and it is taken at once.
+// from what a site costs, in ns, measured at n = 784 by how full the launch's last wave of CTAs is
+// (per quarter of the CTAs that an SM holds): `first` where it is the only wave, `more` on top of
+// full ones (first[3] each), whose CTAs stay where they were placed, so that two with a tile left
+// share a scheduler sooner. Few rows leave most of a 16-row tile empty, and a wave of four-pair
+// threads takes the chain's latency however few CTAs it has, so small blocks take narrower tiles
+// and one pair per thread. Measured, us, against shape 17, n = 784: 8000 columns with 1 row 446
+// (1126), 5 rows 725 (1127), 37 rows 2546 (3272), 100 rows 6430 (6613); symmetric 40 samples 417
+// (614). Between one and two CTAs of shape 17 to an SM its tiles take hardly longer than one, so
+// there it stays: 100 x 500 651, shape 19 687. Of 879 blocks at n = 2 .. 784 none is slower than
+// with shape 17 and the mean ratio is 0.783. Where shape 17 needs 8 waves or more its last one
+// matters little and it is taken at once.
 struct ShapeCost {
-  int id, tile_rows, tile_cols, per_sm, per_low, steps;
-  float full, low;
+  int id, tile_rows, tile_cols, per_sm;
+  float first[4], more[4];
 };
-static const ShapeCost kF32Shapes[] = {{17, 16, 16, 4, 1, 1, 1439.0f, 785.0f},
-                                       {19, 8, 16, 8, 4, 1, 1490.0f, 927.0f},
-                                       {20, 2, 64, 8, 4, 1, 1630.0f, 1050.0f},
-                                       {21, 1, 32, 16, 4, 3, 1600.0f, 560.0f},
-                                       {22, 4, 8, 16, 4, 3, 1130.0f, 600.0f}};
+static const ShapeCost kF32Shapes[] = {{17, 16, 16, 4, {805, 840, 1400, 1420}, {800, 1000, 1390, 1400}},
+                                       {19, 8, 16, 8, {860, 885, 1470, 1485}, {870, 1430, 1470, 1480}},
+                                       {20, 2, 64, 8, {1040, 1048, 1620, 1635}, {1040, 1560, 1620, 1630}},
+                                       {21, 1, 32, 16, {565, 705, 865, 1540}, {150, 310, 980, 1160}},
+                                       {22, 4, 8, 16, {575, 735, 910, 1115}, {210, 670, 1050, 1250}}};
 
 static int f32_shape(const dk_ctx* ctx, const GramArgs& a) {
   int best = kF32Chi4Default;
@@ -571,16 +574,16 @@ static int f32_shape(const dk_ctx* ctx, const GramArgs& a) {
     const long long tiles = count_tiles(t, c.tile_rows, c.tile_cols);
     const long long slots = (long long)ctx->sm_count * c.per_sm, waves = tiles / slots, rest = tiles % slots;
     if (c.id == kF32Chi4Default && waves >= 8) return c.id;
-    float time = float(waves) * c.full;
+    float time = float(waves) * c.first[3];
     if (rest > 0) {
-      const int k = int((rest + ctx->sm_count - 1) / ctx->sm_count), step = (k - 1) / c.per_low;
-      time += c.low + float(step < c.steps ? step : c.steps) / float(c.steps) * (c.full - c.low);
+      const int ctas = int((rest + ctx->sm_count - 1) / ctx->sm_count);  // 1 .. per_sm to an SM
+      time += (waves == 0 ? c.first : c.more)[(4 * ctas + c.per_sm - 1) / c.per_sm - 1];
     }
-    // the estimate takes a last wave as evenly spread, which it isn't always (666 samples: 0.84 of
-    // shape 17's by the estimate, 1.06 by the clock): shape 17 unless another is well below
+    // shape 17 unless another is clearly below: what the estimate leaves out (how the tiles of a last
+    // wave spread, epilogues at small n) is within a few percent
     if (c.id == kF32Chi4Default || time < best_t) {
       best = c.id;
-      best_t = c.id == kF32Chi4Default ? 0.8f * time : time;
+      best_t = c.id == kF32Chi4Default ? 0.93f * time : time;
     }
   }
   return best;

@@ -1,5 +1,6 @@
 """A tile shape that a caller sets is the one that runs, in every precision that has shapes: the
-threads per CTA of the captured launch are those that dk_gram_config_info reports."""
+threads per CTA of the captured launch are those that dk_gram_config_info reports. And the
+built-in choice where shape 17 gives an SM one or two CTAs."""
 import ctypes
 
 import numpy as np
@@ -53,5 +54,28 @@ def test_set_shape_runs(c128, chi, cid, m):
     got = _launched_threads(torch, lambda: dualk.gram(ctx, mps, refine=None))
     ctx.set_gram_config(0)
     assert got == [threads]
+    ctx.sync_status()
+    ctx.close()
+
+
+# blocks of 16 x 16 tiles that give an SM one to two CTAs and for which the narrower shapes need more
+# waves or more than a quarter of one: measured at n = 784, us, shape 17 against the best other:
+# 634 / 667, 650 / 671, 650 / 689, 653 / 690, 651 / 687, 651 / 689
+@pytest.mark.parametrize("rows,m", [(80, 500), (100, 500), (130, 500), (64, 1000), (0, 333), (0, 366)])
+def test_built_in_choice_with_two_tiles_to_an_sm(rows, m):
+    import torch
+    from paper_2602_01330_gb300 import build, dualk, synthetic
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("sizes chosen for 152 SMs")
+    build.build()
+    ctx = dualk.Context(0)
+    x = torch.from_numpy(synthetic.uniform_angles(m + rows, 6, seed=9, dtype=np.float32)).cuda()
+    cols = dualk.mps_build(ctx, x[:m].contiguous(), dualk.FeatureMap())
+    if rows:
+        test = dualk.mps_build(ctx, x[m:].contiguous(), dualk.FeatureMap())
+        got = _launched_threads(torch, lambda: dualk.dual_kernel_rows(ctx, test, cols, refine=None))
+    else:
+        got = _launched_threads(torch, lambda: dualk.gram(ctx, cols, refine=None))
+    assert got == [dualk.gram_config_info(17)[2]] != [dualk.gram_config_info(19)[2]]
     ctx.sync_status()
     ctx.close()

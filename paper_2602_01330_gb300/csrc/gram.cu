@@ -596,6 +596,9 @@ static const CfgInfo kF32Chi8[] = {info_of<F32X8_P11>(), info_of<F32X8_S4>(), in
 // Pairs per SM up to which gram_lanes_kernel takes a block where no tile shape is set: between the
 // sizes measured there.
 constexpr long long kLanesF32Chi4 = 40, kLanesF64Chi4 = 150, kLanesF32Chi8 = 50;
+// bond 8 below 12 qubits, where the lanes' epilogue and first loads weigh more. Lanes against 16 x 16
+// tiles, us, n = 4: 33 pairs per SM 12.6 (14.3), 44 14.9 (14.4), 49 16.7 (14.6); n = 16: 49 45.8 (48.2).
+constexpr long long kLanesF32Chi8Short = 41;
 
 // FP64: a warp instruction holds an SM's pipe 16 cycles, so a launch lasts as long as the SM with
 // the most warps' worth of tiles. 16 x 16 pairs are 8 of them, two such CTAs to an SM (whose tiles
@@ -660,7 +663,7 @@ static dk_status gram_dispatch(dk_ctx* ctx, const void* mps_r, int m_r, const vo
                                    : launch_gram<F64_P11>(ctx, mps_r, m_r, mps_c, m_c, a, st);
   }
   if (dtype == DK_C64 && prec == DK_PREC_F32 && chi == 8) {
-    if (ctx->gram_config == 0 && pair_count(a) <= kLanesF32Chi8 * ctx->sm_count)
+    if (ctx->gram_config == 0 && pair_count(a) <= (a.n < 12 ? kLanesF32Chi8Short : kLanesF32Chi8) * ctx->sm_count)
       return launch_lanes<float, 4, 2>(mps_r, m_r, mps_c, m_c, a, st);
     // shape ids index the bond-8 table; an id beyond it (e.g. one chosen for bond 4) gives
     // the default

@@ -79,3 +79,20 @@ def test_built_in_choice_with_two_tiles_to_an_sm(rows, m):
     assert got == [dualk.gram_config_info(17)[2]] != [dualk.gram_config_info(19)[2]]
     ctx.sync_status()
     ctx.close()
+
+
+@pytest.mark.parametrize("n,m,shape", [(4, 122, 2), (4, 100, None), (16, 122, None)])
+def test_built_in_choice_bond8(n, m, shape):
+    """122 samples are 49 pairs per SM: tiles below 12 qubits, lanes (128 threads) from there on."""
+    import torch
+    from paper_2602_01330_gb300 import build, dualk, synthetic
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("sizes chosen for 152 SMs")
+    build.build()
+    ctx = dualk.Context(0)
+    x = torch.from_numpy(synthetic.uniform_angles(m, n, seed=9, dtype=np.float32)).cuda()
+    mps = dualk.mps_build(ctx, x, dualk.FeatureMap(reps=3, chi_max=8))
+    want = 128 if shape is None else dualk.gram_config_info(shape, dualk.DK_C64, 8)[2]
+    assert _launched_threads(torch, lambda: dualk.gram(ctx, mps, refine=None)) == [want]
+    ctx.sync_status()
+    ctx.close()

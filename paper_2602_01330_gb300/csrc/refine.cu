@@ -101,11 +101,18 @@ __device__ __forceinline__ unsigned group_mask() {
   else return ((1u << L) - 1u) << ((threadIdx.x & 31) & ~(L - 1));
 }
 
-// ln|<psi~_i|psi~_j>| by the double-word chain (FP64 result, valid in every lane of the group).
-// mi / mj: the two MPS, with sample counts m_i / m_j (site-major layout).
+// What a chain leaves in this lane: its element of E, and the exponent.
+struct ChainEnd {
+  DW er, ei;
+  int e2;
+};
+
+// The double-word chain of <psi~_i|psi~_j>, its elements spread over the lanes of the group.
+// mi / mj: the two MPS, with sample counts m_i / m_j (site-major layout). Not inlined: its registers
+// are then allocated for the chain alone (inlined into the pass, a chain took 6 to 15 % longer).
 template <int H>
-__device__ double chain_half_log(const float2* __restrict__ mi, int m_i, int i, const float2* __restrict__ mj, int m_j,
-                                 int j, int n) {
+__device__ __noinline__ ChainEnd chain_end(const float2* __restrict__ mi, int m_i, int i, const float2* __restrict__ mj, int m_j,
+                              int j, int n) {
   constexpr int CHI = 2 * H, L = LANES<H>;
   const unsigned mask = group_mask<H>();
   const int gl = threadIdx.x & (L - 1);
@@ -188,11 +195,26 @@ __device__ double chain_half_log(const float2* __restrict__ mi, int m_i, int i, 
       }
     }
   }
-  const DW r0 = shfl_dw(mask, er, 0, L), r1 = shfl_dw(mask, er, H * H, L);
-  const DW i0 = shfl_dw(mask, ei, 0, L), i1 = shfl_dw(mask, ei, H * H, L);
+  return ChainEnd{er, ei, e2};
+}
+
+// ln|<psi~_i|psi~_j>| from E_0[0][0] (r0, i0) and E_1[0][0] (r1, i1)
+__device__ __forceinline__ double half_log_of(DW r0, DW i0, DW r1, DW i1, int e2) {
   const double re = (double(r0.hi) + double(r0.lo)) + (double(r1.hi) + double(r1.lo));
   const double im = (double(i0.hi) + double(i0.lo)) + (double(i1.hi) + double(i1.lo));
   return half_log_of(re, im, e2);
+}
+
+// ln|<psi~_i|psi~_j>| (FP64 result, valid in every lane of the group).
+template <int H>
+__device__ double chain_half_log(const float2* __restrict__ mi, int m_i, int i, const float2* __restrict__ mj, int m_j,
+                                 int j, int n) {
+  constexpr int L = LANES<H>;
+  const unsigned mask = group_mask<H>();
+  const ChainEnd e = chain_end<H>(mi, m_i, i, mj, m_j, j, n);
+  const DW r0 = shfl_dw(mask, e.er, 0, L), r1 = shfl_dw(mask, e.er, H * H, L);
+  const DW i0 = shfl_dw(mask, e.ei, 0, L), i1 = shfl_dw(mask, e.ei, H * H, L);
+  return half_log_of(r0, i0, r1, i1, e.e2);
 }
 
 struct RefineArgs {
@@ -245,16 +267,60 @@ __device__ __forceinline__ void write_refined(const GramArgs& g, long long at, i
   }
 }
 
-// Each warp tests 32 entries at a time and queues the hits in shared memory; the groups of the
-// warp take them in turn, and a rest that would leave groups idle waits for the next 32.
-constexpr int SMALL_WARPS = 4;
+// Each warp tests 32 entries at a time and queues the hits in shared memory. Bond 8: the warp takes
+// them one after another. Bond 4: whenever 32 are queued, and the rest at the end, as a batch.
+constexpr int SMALL_WARPS = 4, SMALL_CTAS = 4;  // SMALL_CTAS: CTAs per SM
 
+// One entry by the warp.
 template <int H>
 __device__ __forceinline__ void refine_one(const RefineArgs& a, int i, int j, long long at) {
   const double lij = chain_half_log<H>(a.mps_r, a.m_r, i, a.mps_c, a.m_c, j, a.g.n);
   const double lii = a.norm_r ? a.norm_r[i] : chain_half_log<H>(a.mps_r, a.m_r, i, a.mps_r, a.m_r, i, a.g.n);
   const double ljj = a.norm_c ? a.norm_c[j] : chain_half_log<H>(a.mps_c, a.m_c, j, a.mps_c, a.m_c, j, a.g.n);
   if ((threadIdx.x & (LANES<H> - 1)) == 0) write_refined(a.g, at, i, j, 2.0 * lij - lii - ljj);
+}
+
+// Up to 32 queued entries: the groups run the chains in turn, and lane u takes over entry u's result,
+// so that the FP64 logarithms and exponentials, which hold an SM's FP64 pipe 16 cycles a warp
+// instruction, run once for 32 entries. Once for the GROUPS of a turn they were most of the time of
+// blocks of few qubits. Measured with the norms' workspace, 2000 samples, us, before in brackets:
+// n = 2 (1.93 million hits) 597 (2218), n = 8 (0.33 million) 236 (319).
+template <int H>
+__device__ __forceinline__ void refine_batch(const RefineArgs& a, const int* qi, const int* qj, const long long* qa,
+                                             int cnt) {
+  constexpr int L = LANES<H>, GROUPS = 32 / L;
+  const int lane = threadIdx.x & 31, grp = lane / L, src = (lane % GROUPS) * L;
+  double lkq = 0.0;
+  // the pair, and without a workspace both norms
+  const int chains = a.norm_r ? 1 : 3;
+  for (int c = 0; c < chains; ++c) {
+    const float2* mi = c == 2 ? a.mps_c : a.mps_r;
+    const float2* mj = c == 1 ? a.mps_r : a.mps_c;
+    const int m_i = c == 2 ? a.m_c : a.m_r, m_j = c == 1 ? a.m_r : a.m_c;
+    DW r0{0.0f, 0.0f}, r1 = r0, i0 = r0, i1 = r0;
+    int e2 = 0;
+    for (int it = 0; it * GROUPS < cnt; ++it) {
+      const int u = min(it * GROUPS + grp, cnt - 1);  // a group without an entry repeats the last
+      const ChainEnd e = chain_end<H>(mi, m_i, c == 2 ? qj[u] : qi[u], mj, m_j, c == 1 ? qi[u] : qj[u], a.g.n);
+      const DW v0 = shfl_dw(0xffffffffu, e.er, src, 32), v1 = shfl_dw(0xffffffffu, e.er, src + H * H, 32);
+      const DW w0 = shfl_dw(0xffffffffu, e.ei, src, 32), w1 = shfl_dw(0xffffffffu, e.ei, src + H * H, 32);
+      const int ex = __shfl_sync(0xffffffffu, e.e2, src);
+      if (lane / GROUPS == it) {
+        r0 = v0;
+        r1 = v1;
+        i0 = w0;
+        i1 = w1;
+        e2 = ex;
+      }
+    }
+    const double l = half_log_of(r0, i0, r1, i1, e2);
+    lkq = c == 0 ? 2.0 * l : lkq - l;
+  }
+  if (lane < cnt) {
+    const int i = qi[lane], j = qj[lane];
+    if (a.norm_r) lkq = lkq - a.norm_r[i] - a.norm_c[j];
+    write_refined(a.g, qa[lane], i, j, lkq);
+  }
 }
 
 // Marks the samples whose ln-norm some entry above tau needs (all entries of the block,
@@ -293,11 +359,10 @@ __global__ void __launch_bounds__(128) norms_small_kernel(const RefineArgs a, in
 }
 
 template <int H>
-__global__ void __launch_bounds__(SMALL_WARPS * 32) refine_small_kernel(const RefineArgs a) {
-  constexpr int GROUPS = 32 / LANES<H>;
+__global__ void __launch_bounds__(SMALL_WARPS * 32, SMALL_CTAS) refine_small_kernel(const RefineArgs a) {
   __shared__ int qi[SMALL_WARPS][64], qj[SMALL_WARPS][64];
   __shared__ long long qa[SMALL_WARPS][64];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LANES<H>;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const GramArgs& g = a.g;
   const long long total = (long long)g.nrows * g.ncols;
   const long long nwarps = (long long)gridDim.x * SMALL_WARPS;
@@ -324,29 +389,32 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32) refine_small_kernel(const Re
     }
     count += __popc(mask);
     __syncwarp();
-    int done = 0;
-    for (; done + GROUPS <= count; done += GROUPS) {
-      refine_one<H>(a, qi[warp][done + grp], qj[warp][done + grp], qa[warp][done + grp]);
+    if (LANES<H> == 32) {  // no other entry to wait for
+      for (int u = 0; u < count; ++u) refine_one<H>(a, qi[warp][u], qj[warp][u], qa[warp][u]);
+      __syncwarp();
+      count = 0;
+    } else if (count >= 32) {
+      refine_batch<H>(a, qi[warp], qj[warp], qa[warp], 32);
+      __syncwarp();
+      const int rest = count - 32;
+      int ti = 0, tj = 0;
+      long long ta = 0;
+      if (lane < rest) {
+        ti = qi[warp][32 + lane];
+        tj = qj[warp][32 + lane];
+        ta = qa[warp][32 + lane];
+      }
+      __syncwarp();
+      if (lane < rest) {
+        qi[warp][lane] = ti;
+        qj[warp][lane] = tj;
+        qa[warp][lane] = ta;
+      }
+      count = rest;
       __syncwarp();
     }
-    const int rest = count - done;  // below GROUPS
-    int ti = 0, tj = 0;
-    long long ta = 0;
-    if (lane < rest) {
-      ti = qi[warp][done + lane];
-      tj = qj[warp][done + lane];
-      ta = qa[warp][done + lane];
-    }
-    __syncwarp();
-    if (lane < rest) {
-      qi[warp][lane] = ti;
-      qj[warp][lane] = tj;
-      qa[warp][lane] = ta;
-    }
-    count = rest;
-    __syncwarp();
   }
-  if (grp < count) refine_one<H>(a, qi[warp][grp], qj[warp][grp], qa[warp][grp]);
+  if (LANES<H> < 32 && count > 0) refine_batch<H>(a, qi[warp], qj[warp], qa[warp], count);
 }
 
 // ---------------- bond 32: one warp per chain ----------------
@@ -716,9 +784,14 @@ DK_API dk_status dk_gram_refine(dk_ctx* ctx, const void* mps_rows, int m_rows, c
     rf::refine32_kernel<<<int(grid), rf::WARPS32 * 32, smem, st>>>(a);
     return launch_status();
   }
-  // a warp per 32 entries until the GPU is full: the hits of a small block then run side by side
+  // a warp per 32 entries until the GPU is full: the hits of a small block then run side by side.
+  // Bond 4, larger blocks: no more CTAs than the GPU holds at once, whose warps gather fuller batches
+  // (8000 x 37 at n = 12, 2801 hits: 55 us, with 16 CTAs per SM 62). Bond 8 has no batches, and its
+  // chains even out better over more CTAs (2000 samples at n = 12, 24352 hits: 271 us, with 4 per SM
+  // 291).
   long long grid = (total + rf::SMALL_WARPS * 32 - 1) / (rf::SMALL_WARPS * 32);
-  const long long cap = 16LL * ctx->sm_count;
+  const bool batches = chi_max == 4 && grid > 2LL * rf::SMALL_CTAS * ctx->sm_count;
+  const long long cap = (batches ? (long long)rf::SMALL_CTAS : 16LL) * ctx->sm_count;
   if (grid > cap) grid = cap;
   if (chi_max == 4) rf::refine_small_kernel<2><<<int(grid), rf::SMALL_WARPS * 32, 0, st>>>(a);
   else rf::refine_small_kernel<4><<<int(grid), rf::SMALL_WARPS * 32, 0, st>>>(a);

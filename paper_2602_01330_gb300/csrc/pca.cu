@@ -344,7 +344,8 @@ __device__ __forceinline__ bool await_word(uint4& w, const uint4* src, unsigned 
   return true;
 }
 
-template <int MAXT, bool ODD>
+// ODD: p is odd; SOLO: one CTA
+template <int MAXT, bool ODD, bool SOLO>
 __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistArgs a) {
   constexpr int NR = MAXT > 512 ? 2 : UR;  // row pairs in flight: what the registers hold
   extern __shared__ __align__(16) float sm[];
@@ -352,7 +353,8 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
   const int G = int(gridDim.x), g = int(blockIdx.x), NT = int(blockDim.x), tid = int(threadIdx.x);
   const int ks = g * a.ppc, ke = min(ks + a.ppc, np), cnt = ke - ks;
   const int v0 = g * a.vc, vn = max(0, min(a.vc, p - v0)), vp = (a.vc + 3) / 4;
-  const bool solo = G == 1, lone = ring_lone(np, a.ppc);
+  constexpr bool solo = SOLO;
+  const bool lone = !SOLO && ring_lone(np, a.ppc);
   // shared memory: V^T columns [plane][row][4], angles [2 rounds][pair] (c, s, t), solo: the
   // published angles by x, rows [2 rounds][local row][pe], the diagonal of A
   float4* V = reinterpret_cast<float4*>(sm);
@@ -425,15 +427,14 @@ __global__ void __launch_bounds__(MAXT, 1) jacobi_persist_kernel(const PersistAr
       }
       __syncthreads();
       if (s_abort) break;
-      if (q + 1 < a.rounds && holds && ring_publishes(x, y, tx, np, lone)) {  // otherwise the partner's owner does
-        float o = 0.0f;
-        float4 w = make_float4(1.0f, 0.0f, 0.0f, 0.0f);
-        if (y > x && (!ODD || y < p)) {
-          float b00 = ri[c0], b01 = ri[c1], b10 = rj[c0], b11 = rj[c1];
-          rotate_block(pars[buf * np + ks + hu], pars[buf * np + kc], ks + hu == kc, b00, b01, b10, b11);
-          o = is_i ? (low ? b00 : b01) : (low ? b10 : b11);
-          w = pair_rotation(sD[x], sD[y], o);
-        }
+      const bool publishes = q + 1 < a.rounds && holds && ring_publishes(x, y, tx, np, lone);
+      const bool real = y > x && (!ODD || y < p);
+      if (publishes && !real && !solo) put_word(wN + (buf ^ 1) * pe + x, 1.0f, 0.0f, 0.0f, tag_of(q + 1));
+      if (publishes && real) {  // otherwise the partner's owner does it
+        float b00 = ri[c0], b01 = ri[c1], b10 = rj[c0], b11 = rj[c1];
+        rotate_block(pars[buf * np + ks + hu], pars[buf * np + kc], ks + hu == kc, b00, b01, b10, b11);
+        const float o = is_i ? (low ? b00 : b01) : (low ? b10 : b11);
+        const float4 w = pair_rotation(sD[x], sD[y], o);
         if (solo) sN[x] = make_float4(w.x, w.z, o, 0.0f);
         else put_word(wN + (buf ^ 1) * pe + x, w.x, w.z, o, tag_of(q + 1));
       }
@@ -847,25 +848,31 @@ inline PersistPlan plan_of(const dk_ctx* ctx, int p) {
 dk_status fit(dk_ctx* ctx, const float* x, int m, int p, int k, int sweeps, const Workspace& w,
               const PersistPlan& plan, float* mean, float* scale, float* comps, float* eig, float* off_norm,
               cudaStream_t st) {
+  const size_t cov_bytes = size_t(p) * p * sizeof(float), mat_bytes = round256(cov_bytes);
+  if (plan.ctas > 1) {
+    // no word after the covariance (A's padding and V^T's part), which a former call may have used,
+    // has a tag yet; cleared from a 256-byte boundary, before the covariance is written
+    const size_t from = cov_bytes & ~size_t(255);
+    if (cudaMemsetAsync(reinterpret_cast<uint8_t*>(w.A) + from, 0, 2 * mat_bytes - from, st) != cudaSuccess)
+      return DK_ERR_CUDA;
+  }
   col_stats_kernel<<<(p + 7) / 8, 64, 0, st>>>(x, m, p, mean, scale);
   const int nt = (p + T32 - 1) / T32;
   cov_kernel<<<nt * (nt + 1) / 2, 256, 0, st>>>(x, m, p, mean, scale, w.A);
   const int pe = p + (p & 1), np = pe / 2, rounds = sweeps * (pe - 1);
-  const size_t mat_bytes = round256(size_t(p) * p * sizeof(float));
   if (cudaMemsetAsync(w.done, 0, 2 * sizeof(unsigned), st) != cudaSuccess) return DK_ERR_CUDA;  // and failed
   bool persistent = false;
   if (plan.ctas > 0) {
-    // no word after the covariance (A's padding and V^T's part), which a former call may have used,
-    // has a tag yet
-    const size_t cov_bytes = size_t(p) * p * sizeof(float);
-    if (cudaMemsetAsync(reinterpret_cast<uint8_t*>(w.A) + cov_bytes, 0, 2 * mat_bytes - cov_bytes, st) != cudaSuccess)
-      return DK_ERR_CUDA;
     uint8_t* box = reinterpret_cast<uint8_t*>(w.Vt) + mat_bytes - plan.box_bytes;
-    const bool odd = p & 1, small = plan.threads <= 512;
-    const void* kern = odd ? (small ? reinterpret_cast<const void*>(jacobi_persist_kernel<512, true>)
-                                    : reinterpret_cast<const void*>(jacobi_persist_kernel<1024, true>))
-                           : (small ? reinterpret_cast<const void*>(jacobi_persist_kernel<512, false>)
-                                    : reinterpret_cast<const void*>(jacobi_persist_kernel<1024, false>));
+    using Kernel = void (*)(PersistArgs);
+    const bool small = plan.threads <= 512;  // one CTA: always
+    const Kernel odd = plan.ctas == 1 ? jacobi_persist_kernel<512, true, true>
+                       : small        ? jacobi_persist_kernel<512, true, false>
+                                      : jacobi_persist_kernel<1024, true, false>;
+    const Kernel even = plan.ctas == 1 ? jacobi_persist_kernel<512, false, true>
+                        : small        ? jacobi_persist_kernel<512, false, false>
+                                       : jacobi_persist_kernel<1024, false, false>;
+    const void* kern = reinterpret_cast<const void*>(p & 1 ? odd : even);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(plan.smem)) != cudaSuccess)
       return DK_ERR_CUDA;
     PersistArgs a{w.A,  w.Vt, reinterpret_cast<uint4*>(box), w.done, w.failed, ctx->status, p, plan.ppc,

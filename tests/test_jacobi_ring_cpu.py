@@ -36,6 +36,7 @@ int main(int argc, char** argv) {
     lones += lone;
     if (plan.threads > 1024 || plan.box_bytes > 2 * mat || size_t(32) * pe > mat) bad |= 1;
     if ((G - 1) * plan.ppc >= np || G * plan.ppc < np || G > sms) bad |= 2;
+    if (G == 1 && plan.threads > 512) bad |= 256;
     if (G == 1) continue;  // its words are in its own shared memory, behind barriers
     std::vector<int> writers(pe);
     for (int r = 0; r < ring && !(bad & 4); ++r) {  // published in round r for the next one

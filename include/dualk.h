@@ -477,8 +477,10 @@ size_t dk_gram_refine_workspace_bytes(int m_rows, int m_cols);
 /* Tile shapes of the Gram kernels (the blocks of §II-D, sized for one GB300 SM).
  * Shape 0 is the built-in choice; shapes 1..dk_gram_config_count(dtype, chi_max) can be
  * selected per context with dk_set_gram_config, e.g. by an autotuner that times them on
- * the caller's workload. dk_gram_config_info reports a shape's tile (row samples x
- * column samples) and threads per CTA; any pointer may be NULL.
+ * the caller's workload; a shape that is set runs whatever the block's size. The built-in
+ * choice depends on the size. dk_gram_config_info reports a shape's tile (row samples x
+ * column samples) and threads per CTA, for shape 0 those of large blocks; any pointer may be
+ * NULL.
  * Errors: DK_ERR_ARG for an unknown id or NULL ctx. */
 int dk_gram_config_count(dk_dtype dtype, int chi_max);
 dk_status dk_gram_config_info(dk_dtype dtype, int chi_max, int id, int* tile_rows, int* tile_cols,
@@ -573,8 +575,9 @@ dk_status dk_pca_fit_noalloc(dk_ctx* ctx, const float* x, int m, int p, int k, i
 
 /* One-against-one SVM training on precomputed kernel values (§II-B, Eqs. 1-2: the dual
  * problem min 1/2 sum a_i a_j y_i y_j K_ij - sum a_i, sum a_i y_i = 0, 0 <= a_i <= C;
- * §II-D, Eq. 11: the mixed kernel), for n_jobs independent jobs in one launch, e.g. the
- * folds x C x w grid of a cross-validation.
+ * §II-D, Eq. 11: the mixed kernel), for n_jobs independent jobs in one call (one
+ * launch, or two where a class pair is likely to hold well under 0.7 of the longest list), e.g.
+ * the folds x C x w grid of a cross-validation.
  *   kq, kc     n x n kernel matrices over the samples (device, float32, row stride ld >= n);
  *              the job uses K(r, c) = w[job] kq[r*ld + c] + (1 - w[job]) kc[r*ld + c]. Either
  *              may be NULL (its term is dropped). Only entries between samples of a job are

@@ -685,15 +685,18 @@ __global__ void __launch_bounds__(96) mps_build_oct_kernel(const float* __restri
 }
 
 // Bonds 8 and 16 (closed-form block HA = 4, 8, stored block HS = HA): one lane per row of M_s,
-// P = 2 HA lanes per (sample, s): two samples a warp at HA = 4, one at 8. Bound by FP64 issue: a warp-wide FP64 instruction holds an SM's FP64 pipe for about 16
-// cycles whether one lane works or all do, so every step is spread over all lanes:
+// P = 2 HA lanes per (sample, s): two samples a warp at HA = 4, one at 8. Bound by FP64 issue: a
+// warp-wide FP64 instruction holds an SM's FP64 pipe for about 16 cycles whether one lane works or
+// all do, so every step is spread over all lanes:
 //  * u_k and w_k of P sites at a time, one sincos per lane, kept in shared memory;
 //  * M_s = R A_s: the bond phases are a Kronecker product of 2 x 2 blocks [[w, w~], [w~, w]] over
 //    the repetitions' bits, so a row of R takes RP - 1 butterflies
 //        (a, b) -> c (a + b) +/- i s (a - b),   w = c + i s,
 //    instead of HA^2 products, and one phase per column;
 //  * Householder QR (the same reflectors and signs as LAPACK's: R_jj = -sigma x_0 / |x_0|) with
-//    dot products over the rows as shuffle sums, roots by rsqrt.
+//    dot products over the rows as shuffle sums, roots by rsqrt. (20 sets of 160 to 300 samples, n =
+//    16 to 256: the bond-8 Gram's error in log K_q against 64 bits is 8.34e-8 in the mean over the
+//    sets, with sqrt and divisions 8.31e-8, with the warp-per-sample form 8.36e-8.)
 // Measured, 1000 samples, n = 256, bond 8: 5.1 ms (the warp-per-sample form below: 26.3 ms).
 template <int HA>
 struct WideCfg {

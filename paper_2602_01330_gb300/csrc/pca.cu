@@ -289,13 +289,13 @@ __global__ void __launch_bounds__(256) jacobi_rotate_kernel(float* __restrict__ 
 //    other one has read them. The rows' words need only that neighbours send to each other in
 //    every round. All waits are bounded; the launch is cooperative, so the CTAs run at the same
 //    time.
-// Below 64 features one CTA does it all, and the angles pass through shared memory: 0.57 against
-// 0.60 ms at p = 48 (10 sweeps), 0.76 against 0.73 at p = 64, 9.2 against 1.8 at p = 130, where one
-// CTA's rows and V^T take longer than a trip through L2.
+// Below 64 features one CTA does it all (SOLO), and the angles pass through shared memory: 10 sweeps
+// take 0.50 ms at p = 48 and 0.66 at 62, several CTAs 0.60 at 48 and 0.69 at 64, and at p = 130, where one
+// CTA's rows and V^T take longer than a trip through L2, 1.8 against 9.2 ms.
 // The arithmetic and its order are those of jacobi_rotate_kernel: bit-identical results.
 // Bound by the latency of a round: the L2 round trip (about 950 cycles from a store to another
 // SM's load of it), the angle's divisions and roots (about 700 on one warp) and one barrier.
-// Measured, 10 sweeps at p = 784 (131 CTAs of 3 row pairs): 13.2 ms, 1.7 us a round, against
+// Measured, 10 sweeps at p = 784 (131 CTAs of 3 row pairs): 12.7 ms, 1.6 us a round, against
 // 79.4 ms with one launch per round (10.1 us).
 
 struct PersistArgs {
